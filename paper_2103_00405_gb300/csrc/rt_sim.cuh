@@ -31,32 +31,73 @@ __device__ __forceinline__ double i64_to_f64(int64_t h) {
 }
 
 // c * h rounded to nearest-even for a finite c >= 0 and an integer 0 <= h < 2^32,
-// with integer instructions: the 85-bit product of c's significand and h is rounded
-// to 53 bits.  Other operands, and products outside the normal range, use the
+// with integer instructions: the significand of c times h, normalised to 32 bits, is a
+// 96-bit product whose leading bit is known up to one place.  Other operands use the
 // FP64 pipe (identical result: h is exact in binary64).
 __device__ __forceinline__ double mul_rn_pos_u32(double c, int64_t h) {
   if (h == 0) return 0.0;  // c is finite and >= 0
-  const uint64_t bc = (uint64_t)__double_as_longlong(c);
-  const int ec = (int)(bc >> 52);
-  if (h < 0 || h >= (1ll << 32) || ec == 0 || ec >= 0x7FF) return __dmul_rn(c, i64_to_f64(h));
-  const uint64_t cm = (bc & 0x000FFFFFFFFFFFFFull) | (1ull << 52);
-  const uint64_t a0 = (uint64_t)(uint32_t)cm * (uint32_t)h;          // low limb product
-  const uint64_t a1 = (uint64_t)(uint32_t)(cm >> 32) * (uint32_t)h;  // high limb product (< 2^53)
-  const uint64_t lo = a0 + (a1 << 32);
-  const uint64_t hi = (a1 >> 32) + (lo < a0 ? 1u : 0u);  // product = hi 2^64 + lo, < 2^85
-  const int len = hi ? 128 - __clzll(hi) : 64 - __clzll(lo);  // bit length, 53..85
-  const int sh = len - 53;                                    // 0..32
-  if (sh == 0) return __longlong_as_double((long long)(((uint64_t)ec << 52) | (lo & 0x000FFFFFFFFFFFFFull)));
-  uint64_t m = (lo >> sh) | (hi << (64 - sh));
-  const uint64_t rest = lo & ((1ull << sh) - 1), half = 1ull << (sh - 1);
-  m += (rest > half || (rest == half && (m & 1))) ? 1 : 0;
-  int e = ec + sh;
-  if (m >> 53) {
-    m >>= 1;
-    e += 1;
+  const uint32_t ch = (uint32_t)__double2hiint(c), cl = (uint32_t)__double2loint(c);
+  const uint32_t ec = ch >> 20;
+  if ((uint64_t)h >> 32 || ec - 1u >= 2000u) return __dmul_rn(c, i64_to_f64(h));
+  const int s = __clz((int)(uint32_t)h);
+  const uint32_t hs = (uint32_t)h << s;
+  const uint32_t mh = (ch << 11) | 0x80000000u | (cl >> 21), ml = cl << 11;  // significand of c, top bit set
+  const uint64_t p0 = (uint64_t)ml * hs;
+  uint64_t p = (uint64_t)mh * hs + (p0 >> 32);  // the product over 2^32, in [2^62, 2^64)
+  uint32_t st = (uint32_t)p0;
+  const bool top = (int64_t)p < 0;
+  if (!top) {
+    p = (p << 1) | (st >> 31);
+    st <<= 1;
   }
-  if (e >= 0x7FF) return __dmul_rn(c, i64_to_f64(h));
-  return __longlong_as_double((long long)(((uint64_t)e << 52) | (m & 0x000FFFFFFFFFFFFFull)));
+  const uint32_t pl = (uint32_t)p;
+  const bool up = (pl & 0x400u) != 0 && ((pl & 0xBFFu) | st) != 0;  // round bit, and odd or anything below it
+  const uint64_t m = (p >> 11) + (up ? 1u : 0u);  // 53 bits; a carry out of them raises the exponent below
+  return __longlong_as_double((long long)(((uint64_t)(ec + (top ? 31u : 30u) - (uint32_t)s) << 52) + m));
+}
+
+// 1 / x of a float by the special-function unit (at most 1 ulp off)
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// n / d rounded to nearest for n, d > 0, with integer instructions (a binary64 division keeps the
+// FP64 pipe busy for about nine warp instructions of 16 cycles each, and each waits for the one
+// before; this is some 60 integer instructions).  The significand quotient in [1, 2) is taken
+// 30 and then 23 bits at a time, from a reciprocal good to 2^-29; the remainders are exact modulo
+// 2^64, and the last one makes the 54-bit quotient the exact floor.  A quotient of two 53-bit
+// significands is never half-way between two 53-bit numbers, so adding 1 and dropping the last bit
+// rounds it to nearest.  Exponents far out (quotients that may not be normal) take the FP64 pipe.
+// Measured with the product above: Lotka-Volterra ensemble 330 -> 265 ms, 64 Lotka-Volterra paths
+// 359 -> 303 ms, 200-reaction network on warps 84.6 -> 74.8 ms.
+__device__ __forceinline__ double div_rn_pos(double n, double d) {
+  const uint32_t nh = (uint32_t)__double2hiint(n), nl = (uint32_t)__double2loint(n);
+  const uint32_t dh = (uint32_t)__double2hiint(d), dl = (uint32_t)__double2loint(d);
+  const uint32_t en = nh >> 20, ed = dh >> 20;
+  if (!(en - 523u < 1000u && ed - 523u < 1000u)) return __ddiv_rn(n, d);
+  const uint32_t mdh = (dh & 0xFFFFFu) | 0x100000u;
+  const uint64_t mn = ((uint64_t)((nh & 0xFFFFFu) | 0x100000u) << 32) | nl, md = ((uint64_t)mdh << 32) | dl;
+  const bool lt = mn < md;
+  const uint64_t m = lt ? mn << 1 : mn;  // m / md in [1, 2)
+  // r: 2^84 / md in [2^31, 2^32), from a float reciprocal biased below it (by more than the 2^-23 of
+  // the dropped bits and the unit's error, at most 2^-20 in all) and one Newton step; off by -2..4
+  const uint32_t D = __funnelshift_l(dl, mdh, 11);  // md 2^-21, top bit set
+  const float y = fmaxf(rcp_approx(__uint_as_float(0x3F800000u | ((D >> 8) & 0x7FFFFFu))) * 0.9999995f, 0.5f);
+  uint32_t r = (__float_as_uint(y) << 8) | 0x80000000u;
+  r += __umulhi(r, (0x80000000u - __umulhi(r, D)) << 1);
+  const uint32_t q1 = __umulhi((uint32_t)(m >> 22), r) - 8u;    // below the quotient's 30 bits by 4 to 12
+  const uint64_t r1 = (m << 30) - (uint64_t)q1 * md;            // in (0, 2^57)
+  const uint32_t q2 = __umulhi((uint32_t)(r1 >> 25), r) >> 4;   // the next 23 bits, off by -1..1
+  int64_t r2 = (int64_t)((r1 << 23) - (uint64_t)q2 * md);
+  uint64_t q = ((uint64_t)q1 << 23) + q2;
+  if (r2 < 0) {
+    q -= 1;
+    r2 += (int64_t)md;
+  }
+  if (r2 >= (int64_t)md) q += 1;
+  return __longlong_as_double((long long)(((uint64_t)(en - ed + (lt ? 1021u : 1022u)) << 52) + ((q + 1) >> 1)));
 }
 
 // h_k(X) of Eq. 2 for a descriptor {s0, s1}, exact in int64, then a_k = c_k h_k (Eq. 1).
@@ -80,7 +121,7 @@ __device__ __forceinline__ double propensity(int2 rd, double c, XAt x) {
 // Waiting time (P - T) / a of Eq. 25 for a > 0: 0 if no internal time is left.
 __device__ __forceinline__ double waiting_time(double P, double T, double a) {
   const double rem = __dsub_rn(P, T);
-  return dbits(rem) > 0 ? __ddiv_rn(rem, a) : 0.0;
+  return dbits(rem) > 0 ? div_rn_pos(rem, a) : 0.0;
 }
 
 // Time-dependent rates c_k(t) = c_k (1 + beta_k t) (Sec. 6, Eq. 29): with A = c_k h_k(X)
@@ -105,7 +146,7 @@ __device__ __forceinline__ double tdep_integral(double beta, double t, double d)
 
 // The same from an already computed remainder rem = fl(P - T).
 __device__ __forceinline__ double waiting_time_rem(double rem, double a) {
-  return dbits(rem) > 0 ? __ddiv_rn(rem, a) : 0.0;
+  return dbits(rem) > 0 ? div_rn_pos(rem, a) : 0.0;
 }
 
 // An estimate of the quotient rem / a (rem > 0, a > 0) used only to pick which

@@ -39,3 +39,21 @@ def test_draws_equal_the_oracle_over_many_indices():
     lib = oracle.load()
     ref = np.array([lib.oracle_exp1(12345, 3, 7, int(i), 0) for i in range(n)])
     assert np.array_equal(e.cpu().numpy().view(np.int64), ref.view(np.int64))
+
+
+@pytest.mark.parametrize("scale", [1e-310, 1e-200, 1e-37, 1e37, 1e200])
+@pytest.mark.parametrize("m,n", [(1, 1), (3, 2), (4, 4), (7, 6), (14, 7), (40, 10), (600, 60)])
+def test_rates_outside_the_float_range(m, n, scale):
+    """Every second rate scaled far out: estimates, products and quotients at and beyond their ranges."""
+    net = W.pure_birth() if m == 1 else W.random_mass_action(n, m, 900 + m, 0.5)
+    c = net.c.copy()
+    c[::2] *= scale
+    net = net.with_rates(c)
+    x0 = np.full(net.n_species, 40, np.int32)
+    g = api.simulate(api.Network(net), x0, 1e300, 5, seed=3, max_events=150, grad=True)
+    o = oracle.run(net, x0, 1e300, 5, seed=3, max_events=150, want_grad=True, n_threads=4)
+    for key in ("x_final", "n_events", "status", "counts"):
+        assert np.array_equal(g[key].cpu().numpy(), o[key]), key
+    for key in ("t_last", "t_internal", "loglik"):
+        a, b = g[key].cpu().numpy(), o[key]
+        assert ((a.view(np.int64) == b.view(np.int64)) | (np.isnan(a) & np.isnan(b))).all(), key
