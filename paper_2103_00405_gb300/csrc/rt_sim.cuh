@@ -149,6 +149,14 @@ __device__ __forceinline__ double waiting_time_rem(double rem, double a) {
   return dbits(rem) > 0 ? div_rn_pos(rem, a) : 0.0;
 }
 
+// A float estimate of 1 / a, good to 2^-20 + 2^-23: +inf for a = 0 (the channel cannot fire), and 0
+// for an a outside the estimates' range (its waiting-time estimate 0 sends the event to the exact path).
+__device__ __forceinline__ float inv_estimate(double a) {
+  const uint32_t hi = (uint32_t)__double2hiint(a);
+  if (dbits(a) == 0) return __int_as_float(0x7F800000);
+  return hi - (900u << 20) < (240u << 20) ? rcp_approx(__uint_as_float(hi * 8u - 0xC0000000u)) : 0.0f;
+}
+
 // An estimate of the quotient rem / a (rem > 0, a > 0) used only to pick which
 // channel to compute exactly first; the exclusion test below is what is rigorous.
 __device__ __forceinline__ float quot_estimate(double rem, double a) {

@@ -37,6 +37,7 @@ __device__ __forceinline__ void simulate_small(const RunArgs &A, const SmallNet 
   auto xat = [&](int s) { return pick<NMAX>(X, s); };
 
   double P[MAXM], T[MAXM], a[MAXM];
+  float ia[MAXM];  // inv_estimate(a_k)
   int32_t n[MAXM];
   int status = RT_TRAJ_TEND;
   double t = 0.0, ll = 0.0;
@@ -73,6 +74,7 @@ __device__ __forceinline__ void simulate_small(const RunArgs &A, const SmallNet 
     T[k] = 0.0;
     P[k] = 0.0;
     a[k] = 0.0;
+    ia[k] = 0.0f;
   }
   if (bad) {
     status = RT_TRAJ_BAD_X0;
@@ -82,43 +84,49 @@ __device__ __forceinline__ void simulate_small(const RunArgs &A, const SmallNet 
     for (int k = 0; k < MAXM; ++k) {
       P[k] = exp1_draw(A.seed, g, (uint32_t)k, 0u, A.stream_id);
       a[k] = propensity(make_int2(SN.s0[k], SN.s1[k]), SN.c[k], xat);
+      ia[k] = inv_estimate(a[k]);
     }
     const int64_t tend_bits = dbits(A.t_end);
     for (;;) {
-      // Eq. 25-26: waiting times and the first channel to fire (smallest k on ties);
-      // float bounds pick a candidate whose exact quotient is computed first, every
-      // other channel is certified strictly larger or computed exactly as well.
+      // Eq. 25-26: waiting times and the first channel to fire (smallest k on ties).  Float
+      // estimates of the quotients, good to 2^-19, name the winner unless the two smallest lie
+      // within 2^-17 of each other or a value is outside the estimates' range; only the winner's
+      // quotient is then computed exactly.  (Bounds that excluded each other channel by itself cost
+      // three times the instructions: Lotka-Volterra ensemble 265 -> 235 ms, 64 paths 303 -> 270 ms.)
       double rem[MAXM];
-      float ub_min = __int_as_float(0x7F800000);
-      int ks = -1;
+      float m1 = __int_as_float(0x7F800000), m2 = m1;
+      int mu = 0;
+      bool odd = false;
 #pragma unroll
       for (int k = 0; k < MAXM; ++k) {
-        rem[k] = 0.0;
-        if (dbits(a[k]) != 0) {
-          rem[k] = __dsub_rn(P[k], T[k]);
-          const float ub = dbits(rem[k]) > 0 ? quot_estimate(rem[k], a[k]) : 0.0f;
-          if (ks < 0 || ub < ub_min) {
-            ub_min = ub;
-            ks = k;
-          }
+        rem[k] = __dsub_rn(P[k], T[k]);
+        const uint32_t hi = (uint32_t)__double2hiint(rem[k]);
+        odd |= hi - (897u << 20) >= (253u << 20);
+        const float e = __uint_as_float(hi * 8u - 0xC0000000u) * ia[k];  // f32_lower(rem) / a
+        m2 = fminf(m2, fmaxf(m1, e));
+        if (e < m1) {
+          m1 = e;
+          mu = k;
         }
       }
-      int64_t best = kInfBits;
-      int mu = -1;
-      if (ks >= 0) {
-        best = dbits(waiting_time_rem(pick<MAXM>(rem, ks), pick<MAXM>(a, ks)));
-        mu = ks;
-        const float thr = f32_upper(bitsd(best));
-#pragma unroll
-        for (int k = 0; k < MAXM; ++k)
-          if (k != ks && dbits(a[k]) != 0) {
-            if (dbits(rem[k]) > 0 && quot_exceeds(rem[k], a[k], thr)) continue;
-            const int64_t wb = dbits(waiting_time_rem(rem[k], a[k]));
-            if (wb < best || (wb == best && k < mu)) {
-              best = wb;
-              mu = k;
-            }
+      int64_t best;
+      double a_mu = pick<MAXM>(a, mu);
+      if (!odd && m1 >= 1e-30f && m1 < 1e30f && m2 > m1 * 1.00000763f) {
+        best = dbits(div_rn_pos(pick<MAXM>(rem, mu), a_mu));
+      } else {
+        best = kInfBits;
+        mu = -1;
+#pragma unroll 1
+        for (int k = 0; k < MAXM; ++k) {
+          const double ak = pick<MAXM>(a, k);
+          if (dbits(ak) == 0) continue;
+          const int64_t wb = dbits(waiting_time_rem(pick<MAXM>(rem, k), ak));
+          if (wb < best) {
+            best = wb;
+            mu = k;
+            a_mu = ak;
           }
+        }
       }
       if (mu < 0) {
         status = RT_TRAJ_ABSORBED;
@@ -142,8 +150,7 @@ __device__ __forceinline__ void simulate_small(const RunArgs &A, const SmallNet 
         d[s] = SN.delta[0][s];
 #pragma unroll
         for (int k = 1; k < MAXM; ++k) d[s] = (k == mu) ? SN.delta[k][s] : d[s];
-        const long long nx = (long long)X[s] + d[s];
-        over |= (nx > INT_MAX) | (nx < 0);
+        over |= (int)((uint32_t)X[s] + (uint32_t)d[s]) < 0;  // a count past INT_MAX wraps below 0
       }
       if (over) {
         status = RT_TRAJ_OVERFLOW;
@@ -157,12 +164,8 @@ __device__ __forceinline__ void simulate_small(const RunArgs &A, const SmallNet 
       t = tn;
       trace_event(A.out, j, ev, mu, tn);
       // every internal time advances by a_k dt (Eq. 17)
-      double a_mu = 0.0;
 #pragma unroll
-      for (int k = 0; k < MAXM; ++k) {
-        if (k == mu) a_mu = a[k];
-        T[k] = __dadd_rn(T[k], __dmul_rn(a[k], dmin));
-      }
+      for (int k = 0; k < MAXM; ++k) T[k] = __dadd_rn(T[k], __dmul_rn(a[k], dmin));
       if (LL) ll = __dadd_rn(ll, rt_ln(a_mu));
 #pragma unroll
       for (int s = 0; s < NMAX; ++s) X[s] += d[s];
@@ -182,7 +185,10 @@ __device__ __forceinline__ void simulate_small(const RunArgs &A, const SmallNet 
 #pragma unroll
       for (int k = 0; k < MAXM; ++k) {
         if (k == mu) P[k] = Pmu;
-        if ((dm >> k) & 1u) a[k] = propensity(make_int2(SN.s0[k], SN.s1[k]), SN.c[k], xat);
+        if ((dm >> k) & 1u) {
+          a[k] = propensity(make_int2(SN.s0[k], SN.s1[k]), SN.c[k], xat);
+          ia[k] = inv_estimate(a[k]);
+        }
       }
     }
   }
