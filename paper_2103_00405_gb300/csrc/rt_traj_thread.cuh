@@ -252,6 +252,184 @@ __device__ __forceinline__ void simulate_one(const RunArgs &A, const ThreadNet &
   if (A.out.t_last_dev) A.out.t_last_dev[j] = t;
 }
 
+// One thread per trajectory with the channel state in shared memory, columns per thread
+// (element k of thread i at [k * B + i]): P, T, a (binary64) and n.  Kept in registers, the state of
+// 16 channels took 225 of them and left two warps per scheduler, whose 64-cycle FP64 operations then
+// waited for one another; a warp's event moves 6 M doubles through shared memory (12 M cycles), less
+// than its 3 M FP64 instructions take to issue (48 M cycles).  Per event: one pass over the channels
+// for the estimates of the waiting times (as in rt_small.cu: the winner when the two smallest are
+// 2^-17 apart, else the exact minimum), one for T_k += a_k dt, and each lane its own list of changed
+// propensities.
+template <bool LL>
+__device__ __forceinline__ void simulate_mid(const RunArgs &A, const ThreadNet &S, double *state, const int64_t j,
+                                             const int B, const int tend_finite, const int smem_mom) {
+  const int M = A.net.M, N = A.net.N;
+  int *X = S.X + threadIdx.x;  // X[s] lives at X[s * B]
+  double *P = state + threadIdx.x, *T = P + (size_t)M * B, *a = T + (size_t)M * B;
+  int32_t *n = (int32_t *)(state + (size_t)3 * M * B) + threadIdx.x;
+  auto xat = [&](int s) { return X[s * B]; };
+  const uint64_t g = (uint64_t)(A.traj_offset + j);
+  const int32_t *x0 = A.x0 + (A.per_traj_x0 ? j * (int64_t)N : 0);
+  bool bad = false;
+  for (int s = 0; s < N; ++s) {
+    const int v = x0[s];
+    X[s * B] = v;
+    bad |= v < 0;
+  }
+  int status = RT_TRAJ_TEND;
+  double t = 0.0, ll = 0.0;
+  int32_t ev = 0;
+  int64_t gi = 0;
+  double next_g = 0.0;  // time of grid point gi
+
+  // grid sampling: X at grid time gi (right-continuous: events at times <= g included)
+  auto record = [&](int64_t gidx) {
+    if (A.out.grid_dev) {
+      int32_t *gp = A.out.grid_dev + (j * A.G + gidx) * N;
+      for (int s = 0; s < N; ++s) gp[s] = X[s * B];
+    }
+    if (smem_mom) {
+      mom_add(S.mt, gidx, N, xat);
+    } else if (A.out.grid_sum_dev) {
+      for (int s = 0; s < N; ++s) {
+        const long long x = X[s * B];
+        atomicAdd((unsigned long long *)(A.out.grid_sum_dev + gidx * N + s), (unsigned long long)x);
+        if (A.out.grid_sumsq_dev)
+          atomicAdd((unsigned long long *)(A.out.grid_sumsq_dev + gidx * N + s), (unsigned long long)(x * x));
+      }
+      if (A.out.grid_count_dev) atomicAdd((unsigned long long *)(A.out.grid_count_dev + gidx), 1ull);
+    }
+  };
+
+  // initialise (Table 2): first Exp(1) increment per channel, propensities of X(0)
+  for (int k = 0; k < M; ++k) {
+    T[k * B] = 0.0;
+    n[k * B] = 0;
+    P[k * B] = bad ? 0.0 : exp1_draw(A.seed, g, (uint32_t)k, 0u, A.stream_id);
+    a[k * B] = bad ? 0.0 : propensity(S.rd[k], S.c[k], xat);
+  }
+  if (bad) {
+    status = RT_TRAJ_BAD_X0;
+  } else {
+    const int64_t tend_bits = dbits(A.t_end);
+    for (;;) {
+      // Eq. 25-26: waiting times and the first channel to fire (smallest k on ties)
+      float m1 = __int_as_float(0x7F800000), m2 = m1;
+      int mu = 0;
+      bool odd = false;
+#pragma unroll 4
+      for (int k = 0; k < M; ++k) {
+        const double ak = a[k * B];
+        const uint32_t hi = (uint32_t)__double2hiint(__dsub_rn(P[k * B], T[k * B]));
+        odd |= hi - (897u << 20) >= (253u << 20);
+        const float e = __uint_as_float(hi * 8u - 0xC0000000u) * inv_estimate(ak);
+        m2 = fminf(m2, fmaxf(m1, e));
+        if (e < m1) {
+          m1 = e;
+          mu = k;
+        }
+      }
+      int64_t best;
+      double a_mu = a[mu * B];
+      if (!odd && m1 >= 1e-30f && m1 < 1e30f && m2 > m1 * 1.00000763f) {
+        best = dbits(div_rn_pos(__dsub_rn(P[mu * B], T[mu * B]), a_mu));
+      } else {
+        best = kInfBits;
+        mu = -1;
+#pragma unroll 1
+        for (int k = 0; k < M; ++k) {
+          const double ak = a[k * B];
+          if (dbits(ak) == 0) continue;
+          const int64_t wb = dbits(waiting_time(P[k * B], T[k * B], ak));
+          if (wb < best) {
+            best = wb;
+            mu = k;
+            a_mu = ak;
+          }
+        }
+      }
+      if (mu < 0) {
+        status = RT_TRAJ_ABSORBED;
+        break;
+      }
+      const double dmin = bitsd(best);
+      const double tn = __dadd_rn(t, dmin);
+      if (dbits(tn) > tend_bits) {
+        status = RT_TRAJ_TEND;
+        break;
+      }
+      if (ev == A.max_events) {
+        status = RT_TRAJ_MAX_EVENTS;
+        break;
+      }
+      const int vb = S.vp[mu], ve = S.vp[mu + 1];
+      bool over = false;
+      for (int i = vb; i < ve; ++i) {
+        const int2 e = S.vl[i];
+        over |= (int)((uint32_t)X[e.x * B] + (uint32_t)e.y) < 0;  // a count past INT_MAX wraps below 0
+      }
+      if (over) {
+        status = RT_TRAJ_OVERFLOW;
+        break;
+      }
+      while (gi < A.G && dbits(next_g) < dbits(tn)) {
+        record(gi);
+        ++gi;
+        next_g = __dmul_rn(__ll2double_rn(gi), A.sample_dt);
+      }
+      t = tn;
+      trace_event(A.out, j, ev, mu, tn);
+      // every internal time advances by a_k dt (Eq. 17)
+#pragma unroll 4
+      for (int k = 0; k < M; ++k) T[k * B] = __dadd_rn(T[k * B], __dmul_rn(a[k * B], dmin));
+      if (LL) ll = __dadd_rn(ll, rt_ln(a_mu));
+      for (int i = vb; i < ve; ++i) {
+        const int2 e = S.vl[i];
+        X[e.x * B] += e.y;
+      }
+      ++ev;
+      // Eq. 27: only the fired channel draws a new increment
+      const int32_t nmu = n[mu * B] + 1;
+      n[mu * B] = nmu;
+      P[mu * B] = __dadd_rn(P[mu * B], exp1_draw(A.seed, g, (uint32_t)mu, (uint32_t)nmu, A.stream_id));
+      for (uint32_t dm = (uint32_t)S.dep[mu]; dm; dm &= dm - 1) {
+        const int k = __ffs((int)dm) - 1;
+        a[k * B] = propensity(S.rd[k], S.c[k], xat);
+      }
+    }
+  }
+
+  const bool known = status == RT_TRAJ_TEND || status == RT_TRAJ_ABSORBED;
+  for (; gi < A.G; ++gi) {
+    if (known) {
+      record(gi);
+    } else if (A.out.grid_dev) {
+      int32_t *gp = A.out.grid_dev + (j * A.G + gi) * N;
+      for (int s = 0; s < N; ++s) gp[s] = -1;
+    }
+  }
+  if (A.out.loglik_dev || A.out.t_internal_dev) {
+    const double rest = known && tend_finite ? __dsub_rn(A.t_end, t) : 0.0;
+    double sT = 0.0;
+    for (int k = 0; k < M; ++k) {
+      double Tk = T[k * B];
+      if (known && tend_finite) Tk = __dadd_rn(Tk, __dmul_rn(a[k * B], rest));
+      if (A.out.t_internal_dev) A.out.t_internal_dev[j * M + k] = Tk;
+      sT = __dadd_rn(sT, Tk);
+    }
+    if (A.out.loglik_dev)
+      A.out.loglik_dev[j] = status == RT_TRAJ_BAD_X0 ? __longlong_as_double(0x7FF8000000000000ll) : __dsub_rn(ll, sT);
+  }
+  if (A.out.counts_dev)
+    for (int k = 0; k < M; ++k) A.out.counts_dev[j * M + k] = n[k * B];
+  if (A.out.x_final_dev)
+    for (int s = 0; s < N; ++s) A.out.x_final_dev[j * N + s] = X[s * B];
+  trace_tail(A.out, j, ev, 0, 1);
+  if (A.out.n_events_dev) A.out.n_events_dev[j] = ev;
+  if (A.out.status_dev) A.out.status_dev[j] = status;
+  if (A.out.t_last_dev) A.out.t_last_dev[j] = t;
+}
+
 // Table 3's form of the method ("parallel NRRTA", Sec. 5): each channel keeps its relative
 // waiting time w_k; after an event that took dt every propensity is recomputed (no
 // dependency graph) and every other channel's waiting time is rescaled,
