@@ -110,6 +110,9 @@ extern "C" int rt_run(const rt_network *net, const rt_run_params *p, const rt_ou
   }
   switch (mapping) {
     case RT_MAP_THREAD:
+      // left to the library, few trajectories run a warp each
+      if ((!cfg || cfg->mapping == RT_MAP_AUTO) && B <= 0 && lane_mapping_fits(net->dev, a.n_traj))
+        return launch_lane_mapping(a, s);
       // networks of <= 4 reactions and <= 4 species: network in the parameter space, X in registers
       return net->small.ok ? launch_small_mapping(a, net->small, B, s) : launch_thread_mapping(a, B, s);
     case RT_MAP_WARP:

@@ -119,6 +119,8 @@ int launch_tdep_warp_mapping(const RunArgs &a, int lanes_per_traj, cudaStream_t 
 int launch_rescaled_warp_mapping(const RunArgs &a, int lanes_per_traj, cudaStream_t s);
 int launch_small_mapping(const RunArgs &a, const SmallNet &net, int block_threads, cudaStream_t s);
 int thread_mapping_max_m();
+bool lane_mapping_fits(const DevNet &net, int64_t n_traj);
+int launch_lane_mapping(const RunArgs &a, cudaStream_t s);
 size_t bundle_workspace_bytes(const DevNet &net, int64_t n_traj, int ctas_per_traj);
 int launch_warp_mapping(const RunArgs &a, int block_threads, int lanes_per_traj, cudaStream_t s);
 int warp_mapping_max_m();

@@ -72,7 +72,12 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // rounds it to nearest.  Exponents far out (quotients that may not be normal) take the FP64 pipe.
 // Measured with the product above: Lotka-Volterra ensemble 330 -> 265 ms, 64 Lotka-Volterra paths
 // 359 -> 303 ms, 200-reaction network on warps 84.6 -> 74.8 ms.
-__device__ __forceinline__ double div_rn_pos(double n, double d) {
+__device__ __forceinline__ float mant_rcp(double d) {  // of d's significand, its first 24 bits
+  const uint32_t D = __funnelshift_l((uint32_t)__double2loint(d), (uint32_t)__double2hiint(d), 3);
+  return rcp_approx(__uint_as_float(0x3F800000u | (D & 0x7FFFFFu)));
+}
+
+__device__ __forceinline__ double div_rn_pos(double n, double d, float rcp_d) {  // rcp_d = mant_rcp(d)
   const uint32_t nh = (uint32_t)__double2hiint(n), nl = (uint32_t)__double2loint(n);
   const uint32_t dh = (uint32_t)__double2hiint(d), dl = (uint32_t)__double2loint(d);
   const uint32_t en = nh >> 20, ed = dh >> 20;
@@ -84,7 +89,7 @@ __device__ __forceinline__ double div_rn_pos(double n, double d) {
   // r: 2^84 / md in [2^31, 2^32), from a float reciprocal biased below it (by more than the 2^-23 of
   // the dropped bits and the unit's error, at most 2^-20 in all) and one Newton step; off by -2..4
   const uint32_t D = __funnelshift_l(dl, mdh, 11);  // md 2^-21, top bit set
-  const float y = fmaxf(rcp_approx(__uint_as_float(0x3F800000u | ((D >> 8) & 0x7FFFFFu))) * 0.9999995f, 0.5f);
+  const float y = fmaxf(rcp_d * 0.9999995f, 0.5f);
   uint32_t r = (__float_as_uint(y) << 8) | 0x80000000u;
   r += __umulhi(r, (0x80000000u - __umulhi(r, D)) << 1);
   const uint32_t q1 = __umulhi((uint32_t)(m >> 22), r) - 8u;    // below the quotient's 30 bits by 4 to 12
@@ -99,6 +104,8 @@ __device__ __forceinline__ double div_rn_pos(double n, double d) {
   if (r2 >= (int64_t)md) q += 1;
   return __longlong_as_double((long long)(((uint64_t)(en - ed + (lt ? 1021u : 1022u)) << 52) + ((q + 1) >> 1)));
 }
+
+__device__ __forceinline__ double div_rn_pos(double n, double d) { return div_rn_pos(n, d, mant_rcp(d)); }
 
 // h_k(X) of Eq. 2 for a descriptor {s0, s1}, exact in int64, then a_k = c_k h_k (Eq. 1).
 // IMUL: the product on integer instructions (faster where the FP64 pipe is the
