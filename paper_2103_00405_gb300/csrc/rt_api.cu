@@ -195,22 +195,39 @@ extern "C" int rt_philox(int64_t count, const uint32_t *ctr, uint32_t key0, uint
 }
 
 // ---------------------------------------------------------------------------
-// Backward: grad_c[k] = sum_j g_j (n_jk - T_jk) / c_k.  One block per 32
-// channels; each of 32 row lanes sums every 32nd trajectory in index order,
-// then the 32 lane sums are added in lane order: a fixed summation order.
+// Backward: grad_c[k] = sum_j g_j (n_jk - T_jk) / c_k.  Each of 32 row lanes sums
+// every 32nd trajectory in index order, then the 32 lane sums are added in lane
+// order: a fixed summation order.  Four channels (one 32-byte sector of T) per
+// block, so that 64 channels fill 16 SMs; each lane forms eight terms before it
+// adds them in order, so only the additions wait for one another, and the
+// quotient is the integer one.  (32 channels per block and the FP64 division:
+// 6.8 ms for 65536 trajectories of 64 reactions.)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_loglik_backward(int32_t M, int64_t n_traj, const double *g,
-                                                          const int32_t *counts, const double *Tend,
-                                                          const double *c, double *grad) {
-  __shared__ double part[32][33];
-  const int col = blockIdx.x * 32 + threadIdx.x;
+constexpr int kBackCols = 4, kBackAhead = 8;
+
+__global__ void __launch_bounds__(kBackCols * 32) k_loglik_backward(int32_t M, int64_t n_traj, const double *g,
+                                                                   const int32_t *counts, const double *Tend,
+                                                                   const double *c, double *grad) {
+  __shared__ double part[32][kBackCols];
+  const int col = blockIdx.x * kBackCols + threadIdx.x;
   double s = 0.0;
   if (col < M) {
     const double ck = c[col];
-    for (int64_t j = threadIdx.y; j < n_traj; j += 32) {
+    auto term = [&](int64_t j) {
       const double d = __dsub_rn(__int2double_rn(counts[j * M + col]), Tend[j * M + col]);
-      s = __dadd_rn(s, __dmul_rn(g[j], __ddiv_rn(d, ck)));
+      // d / c_k: the sign of d on the quotient of the magnitudes (c_k >= 0)
+      const double q = dbits(d) << 1 ? div_rn_pos(fabs(d), ck) : __ddiv_rn(d, ck);
+      return __dmul_rn(g[j], copysign(q, d));
+    };
+    int64_t j = threadIdx.y;
+    for (; j + 32 * (kBackAhead - 1) < n_traj; j += 32 * kBackAhead) {
+      double v[kBackAhead];
+#pragma unroll
+      for (int i = 0; i < kBackAhead; ++i) v[i] = term(j + 32 * i);
+#pragma unroll
+      for (int i = 0; i < kBackAhead; ++i) s = __dadd_rn(s, v[i]);
     }
+    for (; j < n_traj; j += 32) s = __dadd_rn(s, term(j));
   }
   part[threadIdx.y][threadIdx.x] = s;
   __syncthreads();
@@ -230,8 +247,8 @@ extern "C" int rt_loglik_backward(const rt_network *net, int64_t n_traj, const d
   int rc = check_device(net);
   if (rc) return rc;
   const int M = net->dev.M;
-  dim3 block(32, 32);
-  k_loglik_backward<<<(M + 31) / 32, block, 0, (cudaStream_t)stream>>>(M, n_traj, grad_ll, counts, Tend, net->dev.c0,
+  dim3 block(kBackCols, 32);
+  k_loglik_backward<<<(M + kBackCols - 1) / kBackCols, block, 0, (cudaStream_t)stream>>>(M, n_traj, grad_ll, counts, Tend, net->dev.c0,
                                                                      grad_c);
   const cudaError_t err = cudaGetLastError();
   return err == cudaSuccess ? RT_OK : set_error(RT_ERR_CUDA, "%s", cudaGetErrorString(err));
