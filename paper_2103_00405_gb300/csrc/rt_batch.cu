@@ -27,6 +27,9 @@ namespace rt {
 
 enum { CLS_THREAD = 0, CLS_WARP = 1, CLS_BLOCK = 2 };
 
+constexpr size_t kBatchSmem = 100 * 1024;  // shared memory of a block with which two fit on an SM
+constexpr size_t kBatchSmemMax = 226 * 1024;  // of the 227 KB a block can have
+
 struct BNet {
   DevNet d;
   int64_t xoff;  // first species of this network in the packed x0 / x_final rows
@@ -50,7 +53,9 @@ struct BatchArgs {
   int32_t max_events;
   uint64_t seed;
   rt_batch_outputs out;
-  int maxN_thread, maxN_warp, maxM_block, maxN_block;
+  int maxN_thread, maxM_block, maxN_block;
+  size_t warp_bytes;   // shared memory of one warp-class trajectory
+  int warp_task;       // warp-class trajectories per task
 };
 
 __device__ __forceinline__ RunArgs item_args(const BatchArgs &B, int net_index, const BNet &bn) {
@@ -120,21 +125,21 @@ __global__ void __launch_bounds__(512, 2) k_batch(const BatchArgs B) {
     }
     t -= B.tasks[CLS_BLOCK];
     if (t < B.tasks[CLS_WARP]) {
-      // W warp-class trajectories
-      const int64_t f = t * W + warp;
-      if (f < (int64_t)B.n_cls[CLS_WARP] * B.n_traj) {
+      // warp_task warp-class trajectories
+      const int64_t f = t * B.warp_task + warp;
+      if (warp < B.warp_task && f < (int64_t)B.n_cls[CLS_WARP] * B.n_traj) {
         const int ni = B.order[CLS_WARP][f / B.n_traj];
         const int64_t j = f % B.n_traj;
         const BNet bn = B.nets[ni];
         const RunArgs A = item_args(B, ni, bn);
-        const WarpNet net{bn.d.M, bn.d.N, bn.d.n_vnz, bn.d.rdesc, bn.d.c, bn.d.vptr, bn.d.vlist, bn.d.depw};
-        int *X = (int *)smem + warp * B.maxN_warp;
+        const WarpNet net{bn.d.M, bn.d.N, bn.d.rdesc, bn.d.c, bn.d.vptr, bn.d.vlist, bn.d.dptr, bn.d.dlist, nullptr};
+        unsigned char *X = smem + (size_t)warp * B.warp_bytes;
         const int tf = isfinite(A.t_end) ? 1 : 0;
         switch (bn.R) {
-          case 1: warp_trajectories<1, 32, LL>(A, net, X, nullptr, j, tf); break;
-          case 2: warp_trajectories<2, 32, LL>(A, net, X, nullptr, j, tf); break;
-          case 4: warp_trajectories<4, 32, LL>(A, net, X, nullptr, j, tf); break;
-          default: warp_trajectories<8, 32, LL>(A, net, X, nullptr, j, tf); break;
+          case 1: warp_trajectories<1, 32, LL, false>(A, net, X, nullptr, j, tf); break;
+          case 2: warp_trajectories<2, 32, LL, false>(A, net, X, nullptr, j, tf); break;
+          case 4: warp_trajectories<4, 32, LL, false>(A, net, X, nullptr, j, tf); break;
+          default: warp_trajectories<8, 32, LL, false>(A, net, X, nullptr, j, tf); break;
         }
       }
       continue;
@@ -177,7 +182,9 @@ struct rt_batch {
   int32_t n_cls[3] = {0, 0, 0};
   int64_t total_species = 0, total_reactions = 0;
   rt_batch_policy policy;
-  int maxN_thread = 1, maxN_warp = 1, maxM_block = 1, maxN_block = 1;
+  int maxN_thread = 1, maxM_block = 1, maxN_block = 1;
+  size_t warp_bytes = 0;
+  int warp_task = 1;
   size_t smem = 0;
   int grid = 0;
 };
@@ -237,7 +244,7 @@ extern "C" int rt_batch_create(int32_t n_nets, const rt_network *const *nets, co
       b->maxM_block = std::max(b->maxM_block, M);
       b->maxN_block = std::max(b->maxN_block, N);
     }
-    if (cls == CLS_WARP) b->maxN_warp = std::max(b->maxN_warp, N);
+    if (cls == CLS_WARP) b->warp_bytes = std::max(b->warp_bytes, warp_seg_bytes(M, N, 32));
     if (cls == CLS_THREAD) b->maxN_thread = std::max(b->maxN_thread, N);
     hn[i].xoff = b->total_species;
     hn[i].moff = b->total_reactions;
@@ -285,9 +292,6 @@ extern "C" int rt_batch_create(int32_t n_nets, const rt_network *const *nets, co
     d.sptr = (const int32_t *)(db + g->off_sptr);
     d.slist = (const int32_t *)(db + g->off_slist);
     d.depmask = g->dev.depmask ? (const uint64_t *)(db + g->off_dep) : nullptr;
-    d.depw = g->dev.depw ? (const uint8_t *)(db + g->off_depw) : nullptr;
-    d.depw16 = g->dev.depw16 ? (const uint8_t *)(db + g->off_depw16) : nullptr;
-    d.depw8 = g->dev.depw8 ? (const uint8_t *)(db + g->off_depw8) : nullptr;
     d.vdep = g->dev.vdep ? (const int4 *)(db + g->off_vdep) : nullptr;
     d.dptr = g->dev.dptr ? (const int32_t *)(db + g->off_dptr) : nullptr;
     d.dlist = g->dev.dptr ? (const int32_t *)(db + g->off_dlist) : nullptr;
@@ -309,10 +313,14 @@ extern "C" int rt_batch_create(int32_t n_nets, const rt_network *const *nets, co
   // shared memory: the largest of the three uses (a block runs one task at a time)
   const int BT = pol.block_threads;
   const size_t s_block = b->n_cls[CLS_BLOCK] ? block_scratch_bytes(b->maxM_block, b->maxN_block, BT) : 0;
-  const size_t s_warp = (size_t)(BT / 32) * b->maxN_warp * 4;
   const size_t s_thread = (size_t)BT * b->maxN_thread * 4;
+  // warp-class trajectories per task: one per warp of the block, as far as two blocks per SM can hold
+  // their state (or as the other classes' shared memory allows anyway)
+  const size_t room = std::max({s_block, s_thread, kBatchSmem});
+  b->warp_task = (int)std::min<size_t>(BT / 32, std::max<size_t>(1, b->warp_bytes ? room / b->warp_bytes : 1));
+  const size_t s_warp = b->n_cls[CLS_WARP] ? b->warp_task * b->warp_bytes : 0;
   b->smem = std::max({s_block, s_warp, s_thread, (size_t)16});
-  if (b->smem > 200 * 1024) {
+  if (b->smem > kBatchSmemMax) {
     const size_t need = b->smem;
     cudaFree(b->arena);
     delete b;
@@ -371,7 +379,7 @@ extern "C" int rt_batch_run(rt_batch *b, const int32_t *x0_dev, const double *t_
   A.n_traj = n_traj_per_net;
   const int BT = b->policy.block_threads;
   A.tasks[CLS_BLOCK] = (int64_t)b->n_cls[CLS_BLOCK] * n_traj_per_net;
-  A.tasks[CLS_WARP] = ((int64_t)b->n_cls[CLS_WARP] * n_traj_per_net + BT / 32 - 1) / (BT / 32);
+  A.tasks[CLS_WARP] = ((int64_t)b->n_cls[CLS_WARP] * n_traj_per_net + b->warp_task - 1) / b->warp_task;
   A.tasks[CLS_THREAD] = ((int64_t)b->n_cls[CLS_THREAD] * n_traj_per_net + BT - 1) / BT;
   A.n_tasks = A.tasks[0] + A.tasks[1] + A.tasks[2];
   A.counter = b->d_counter;
@@ -382,7 +390,8 @@ extern "C" int rt_batch_run(rt_batch *b, const int32_t *x0_dev, const double *t_
   memset(&A.out, 0, sizeof(A.out));
   if (outputs) A.out = *outputs;
   A.maxN_thread = b->maxN_thread;
-  A.maxN_warp = b->maxN_warp;
+  A.warp_bytes = b->warp_bytes;
+  A.warp_task = b->warp_task;
   A.maxM_block = b->maxM_block;
   A.maxN_block = b->maxN_block;
   cudaStream_t s = (cudaStream_t)stream;

@@ -29,16 +29,13 @@ struct DevNet {
   const int32_t *sptr;     // [N+1] reactions with species s as a reactant: slist[sptr[s]..sptr[s+1])
   const int32_t *slist;
   const uint64_t *depmask; // [M] (M <= 64 only) bit k: firing changes a species channel k reads
-  const uint8_t *depw;     // [M][32] (M <= 256 only) bit r of depw[mu*32 + l]: channel l + 32 r depends on mu
-  const uint8_t *depw16;   // [M][16] (M <= 128 only) the same for 16-lane segments: channel l + 16 r
-  const uint8_t *depw8;    // [M][8]  (M <= 64 only)  the same for 8-lane segments: channel l + 8 r
   const double *beta;      // [M] rate slopes, c_k(t) = c_k (1 + beta_k t); null for constant rates
   const int4 *vdep;        // [M][3] per reaction, when it fits (else null): its net change packed in
                            // 4 words (species << 8) | (delta & 0xFF), unused words 0; then for each
                            // changed species the begin and the length of its reader list in slist
   const int32_t *dptr;     // [M+1] (M <= kDepListMaxM, else null) the channels whose propensity
   const int32_t *dlist;    // reaction k's firing changes: dlist[dptr[k]..dptr[k+1]) (the reader
-                           // lists of its changed species, concatenated; repeats possible)
+                           // lists of its changed species, merged)
 };
 
 // Networks up to this many reactions get the per-reaction dependent lists (dptr/dlist).
@@ -73,7 +70,6 @@ struct rt_network {
   size_t off_rdesc = 0, off_c = 0, off_c0 = 0, off_vptr = 0, off_vlist = 0, off_sptr = 0, off_slist = 0, off_dep = 0;
   std::vector<double> c_host;  // the network's rates (host copy)
   double *beta_dev = nullptr;  // rate slopes on the device (rt_network_set_rate_slopes), or null
-  size_t off_depw = 0, off_depw16 = 0, off_depw8 = 0;
   size_t off_vdep = 0, off_dptr = 0, off_dlist = 0;
   rt::SmallNet small = {};  // filled when M <= kSmallM and N <= kSmallN
 };

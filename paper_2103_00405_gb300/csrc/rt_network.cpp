@@ -168,22 +168,6 @@ extern "C" int rt_network_create(int32_t N, int32_t M, int64_t n_reac_nz, const 
       for (int32_t i = vptr[k]; i < vptr[k + 1]; i++)
         for (int32_t q = sptr[vlist[i].x]; q < sptr[vlist[i].x + 1]; q++) depmask[k] |= 1ull << slist[q];
   }
-  // per reaction and lane of a G-lane segment: which of the lane's channels (l + G r, r < 8)
-  // read a changed species
-  auto dep_bytes = [&](int G) {
-    std::vector<uint8_t> d((size_t)M * G, 0);
-    for (int32_t k = 0; k < M; k++)
-      for (int32_t i = vptr[k]; i < vptr[k + 1]; i++)
-        for (int32_t q = sptr[vlist[i].x]; q < sptr[vlist[i].x + 1]; q++) {
-          const int32_t ch = slist[q];
-          d[(size_t)k * G + (ch % G)] |= (uint8_t)(1u << (ch / G));
-        }
-    return d;
-  };
-  std::vector<uint8_t> depw, depw16, depw8;
-  if (M <= 256) depw = dep_bytes(32);
-  if (M <= 128) depw16 = dep_bytes(16);
-  if (M <= 64) depw8 = dep_bytes(8);
   // per reaction in 48 bytes, when every reaction changes at most 4 species by -128..127 and
   // N < 2^24: its packed net change and the reader lists of the species it changes (one load
   // per fired reaction in the tree mapping)
@@ -207,14 +191,19 @@ extern "C" int rt_network_create(int32_t N, int32_t M, int64_t n_reac_nz, const 
       }
     }
   }
-  // per reaction the channels its firing touches: the reader lists of its changed species,
-  // concatenated (small and mid-size networks; the block routine marks them from one list)
+  // per reaction the channels its firing touches, each once: the reader lists of its changed
+  // species, merged (small and mid-size networks)
   std::vector<int32_t> dptr, dlist;
   if (M <= kDepListMaxM) {
     dptr.assign((size_t)M + 1, 0);
+    std::vector<int32_t> seen(M, -1);  // the last reaction whose list has this channel
     for (int32_t k = 0; k < M; k++) {
       for (int32_t i = vptr[k]; i < vptr[k + 1]; i++)
-        for (int32_t q = sptr[vlist[i].x]; q < sptr[vlist[i].x + 1]; q++) dlist.push_back(slist[q]);
+        for (int32_t q = sptr[vlist[i].x]; q < sptr[vlist[i].x + 1]; q++)
+          if (seen[slist[q]] != k) {
+            seen[slist[q]] = k;
+            dlist.push_back(slist[q]);
+          }
       dptr[(size_t)k + 1] = (int32_t)dlist.size();
     }
   }
@@ -233,9 +222,6 @@ extern "C" int rt_network_create(int32_t N, int32_t M, int64_t n_reac_nz, const 
   g->off_sptr = off; off = align_up(off + sizeof(int32_t) * (N + 1), 256);
   g->off_slist = off; off = align_up(off + sizeof(int32_t) * std::max<size_t>(1, slist.size()), 256);
   g->off_dep = off; off = align_up(off + sizeof(uint64_t) * std::max<size_t>(1, depmask.size()), 256);
-  g->off_depw = off; off = align_up(off + std::max<size_t>(1, depw.size()), 256);
-  g->off_depw16 = off; off = align_up(off + std::max<size_t>(1, depw16.size()), 256);
-  g->off_depw8 = off; off = align_up(off + std::max<size_t>(1, depw8.size()), 256);
   g->off_vdep = off; off = align_up(off + sizeof(int4) * std::max<size_t>(1, vdep.size()), 256);
   g->off_dptr = off; off = align_up(off + sizeof(int32_t) * std::max<size_t>(1, dptr.size()), 256);
   g->off_dlist = off; off = align_up(off + sizeof(int32_t) * std::max<size_t>(1, dlist.size()), 256);
@@ -251,9 +237,6 @@ extern "C" int rt_network_create(int32_t N, int32_t M, int64_t n_reac_nz, const 
   memcpy(hb + g->off_sptr, sptr.data(), sizeof(int32_t) * (N + 1));
   if (!slist.empty()) memcpy(hb + g->off_slist, slist.data(), sizeof(int32_t) * slist.size());
   if (!depmask.empty()) memcpy(hb + g->off_dep, depmask.data(), sizeof(uint64_t) * depmask.size());
-  if (!depw.empty()) memcpy(hb + g->off_depw, depw.data(), depw.size());
-  if (!depw16.empty()) memcpy(hb + g->off_depw16, depw16.data(), depw16.size());
-  if (!depw8.empty()) memcpy(hb + g->off_depw8, depw8.data(), depw8.size());
   if (!vdep.empty()) memcpy(hb + g->off_vdep, vdep.data(), sizeof(int4) * vdep.size());
   if (!dptr.empty()) memcpy(hb + g->off_dptr, dptr.data(), sizeof(int32_t) * dptr.size());
   if (!dlist.empty()) memcpy(hb + g->off_dlist, dlist.data(), sizeof(int32_t) * dlist.size());
@@ -285,9 +268,6 @@ extern "C" int rt_network_create(int32_t N, int32_t M, int64_t n_reac_nz, const 
   d.sptr = (const int32_t *)(db + g->off_sptr);
   d.slist = (const int32_t *)(db + g->off_slist);
   d.depmask = M <= 64 ? (const uint64_t *)(db + g->off_dep) : nullptr;
-  d.depw = M <= 256 ? (const uint8_t *)(db + g->off_depw) : nullptr;
-  d.depw16 = M <= 128 ? (const uint8_t *)(db + g->off_depw16) : nullptr;
-  d.depw8 = M <= 64 ? (const uint8_t *)(db + g->off_depw8) : nullptr;
   d.vdep = vdep.empty() ? nullptr : (const int4 *)(db + g->off_vdep);
   d.dptr = dptr.empty() ? nullptr : (const int32_t *)(db + g->off_dptr);
   d.dlist = dptr.empty() ? nullptr : (const int32_t *)(db + g->off_dlist);

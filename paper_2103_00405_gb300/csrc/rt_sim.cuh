@@ -63,6 +63,12 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // n / d rounded to nearest for n, d > 0, with integer instructions (a binary64 division keeps the
 // FP64 pipe busy for about nine warp instructions of 16 cycles each, and each waits for the one
 // before; this is some 60 integer instructions).  The significand quotient in [1, 2) is taken
@@ -174,6 +180,42 @@ __device__ __forceinline__ float quot_estimate(double rem, double a) {
 __device__ __forceinline__ bool quot_exceeds(double rem, double a, float thr) {
   return f32_lower(rem) > __fmul_ru(thr, f32_upper(a));
 }
+
+// Float intervals of the waiting time (P - T) / a, kept per channel as {upper_P(P), inv_upper(a)}.
+// A float >= P + 2^-125 (the term covers the floor of T's bound below); +inf from 2^127 on, where
+// the interval becomes NaN and the channel is computed exactly.
+__device__ __forceinline__ float upper_P(double P) {
+  const uint32_t hi = (uint32_t)__double2hiint(P);
+  return hi >= (1150u << 20) ? __int_as_float(0x7F800000) : __fadd_ru(f32_upper(P), 0x1p-125f);
+}
+
+// An upper bound of 1 / a, at most 2^-18 above it; +inf for a = 0 (the interval is at +inf); NaN where
+// the float arithmetic could leave its range: never excluded, and ignored by the threshold.
+__device__ __forceinline__ float inv_upper(double a) {
+  const uint32_t hi = (uint32_t)__double2hiint(a);
+  if (dbits(a) == 0) return __int_as_float(0x7F800000);
+  return hi - (900u << 20) < (240u << 20) ? rcp_approx(__uint_as_float(hi * 8u - 0xC0000000u)) * 1.00000191f
+                                          : __int_as_float(0x7FC00000);
+}
+
+// rem >= P - T >= rem - slack from the kept bound of P (the bound's excess is below 2^-19 P, that of
+// T's float below 2^-20 T, and T exceeds P by a rounding at most).
+__device__ __forceinline__ float rem_upper(float Pu, double T) {
+  const uint32_t hi = max((uint32_t)__double2hiint(T), 897u << 20);
+  return __fsub_ru(Pu, __uint_as_float(hi * 8u - 0xC0000000u));
+}
+__device__ __forceinline__ float rem_slack(float Pu) { return __fmaf_ru(Pu, 0x1p-18f, 0x1p-120f); }
+
+// The upper end; lo is the lower end up to the factor that interval_threshold allows for.
+__device__ __forceinline__ float wait_interval(float2 b, double T, float &lo) {
+  const float rem = rem_upper(b.x, T);
+  lo = __fmul_rd(__fsub_rd(rem, rem_slack(b.x)), b.y);
+  return __fmul_ru(rem, b.y);
+}
+
+// A channel with lo above this has a waiting time above ub: the reciprocal's 2^-18 and the roundings
+// of the exact operations are below 2^-17.
+__device__ __forceinline__ float interval_threshold(float ub) { return __fmul_ru(fmaxf(ub, 0.0f), 1.00000763f); }
 
 // An estimate of (P - T) / a used only to choose the candidate that is computed
 // exactly first (any choice gives the same, exact result).

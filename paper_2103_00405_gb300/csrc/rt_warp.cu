@@ -1,6 +1,7 @@
 // rt_warp.cu -- warp segments per trajectory (8, 16 or 32 lanes each) for networks of up
-// to 256 reactions: the single-network kernel around warp_trajectories (rt_traj_warp.cuh);
-// the network is copied to shared memory once per block of four warps.
+// to 256 reactions: the single-network kernel around warp_trajectories (rt_traj_warp.cuh),
+// for constant and time-dependent rates; the network is copied to shared memory once per
+// block.  Beside it Table 3's form with a lane per channel.
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -10,7 +11,8 @@
 
 namespace rt {
 
-constexpr int kWarpBlock = 128;  // 4 warps per block
+constexpr int kWarpBlock = 128;                 // at most 4 warps per block
+constexpr size_t kWarpSmemMax = 226 * 1024;  // of the 227 KB a block can have
 
 static size_t warp_moment_bytes(const RunArgs &a) {
   if (!a.out.grid_sum_dev) return 0;
@@ -18,40 +20,49 @@ static size_t warp_moment_bytes(const RunArgs &a) {
   return b <= 64 * 1024 ? b : 0;
 }
 
-// Eight channels per lane need about 150 registers; bounding them to 128 keeps four blocks
-// (16 warps) per SM.
-template <int R, int G, bool LL>
-__global__ void __launch_bounds__(kWarpBlock, R >= 8 ? 4 : 1)
+// Start of the trajectories' state in a block's shared memory, after the network's tables and the
+// moment table.
+__host__ __device__ inline size_t warp_state_off(int M, int nv, int64_t nmom, bool td) {
+  const size_t b = (size_t)M * (8 + 8 + (td ? 8 : 0)) + (size_t)nv * 8 + (size_t)nmom * 8 + (size_t)(M + 1) * 4;
+  return (b + 127) / 128 * 128;
+}
+
+// Registers bounded (80) for six blocks, 24 warps, per SM.  Against the state in registers (128, 16 warps):
+// 65536 trajectories of 64 reactions with likelihood and gradient 350 -> 186 ms, 10000 trajectories of 200
+// reactions with moments 74.8 -> 51.8 ms; time-dependent rates against every root exactly with one
+// trajectory per warp: 10000 trajectories of 48 reactions 83 -> 26 ms.
+template <int R, int G, bool LL, bool TD>
+__global__ void __launch_bounds__(kWarpBlock, 6)
     k_ens_warp(const RunArgs A, const int tend_finite, const int use_mom) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   constexpr int S = 32 / G;  // trajectories per warp
   const DevNet &d = A.net;
-  const int M = d.M, N = d.N, nv = d.n_vnz;
-  const uint8_t *depg = G == 8 ? d.depw8 : G == 16 ? d.depw16 : d.depw;
-  // carve: c[M], rd[M], vl[nv], moments, vp[M+1], dep[M*G], X[warps * S][N]
+  const int M = d.M, N = d.N, nv = TD ? 0 : d.n_vnz;
+  // carve: c[M], beta[M] (TD), rd[M], vl[nv], moments, vp[M+1], the trajectories
   double *s_c = (double *)smem;
-  int2 *s_rd = (int2 *)(s_c + M);
+  double *s_beta = s_c + M;
+  int2 *s_rd = (int2 *)(s_beta + (TD ? M : 0));
   int2 *s_vl = s_rd + M;
   unsigned long long *s_mom = (unsigned long long *)(s_vl + nv);
   const int64_t GN = A.G * N;
   const int64_t nmom = use_mom ? 2 * GN + A.G : 0;
   int *s_vp = (int *)(s_mom + nmom);
-  uint8_t *s_dep = (uint8_t *)(s_vp + M + 1);
-  int *s_X = (int *)(s_dep + (((size_t)M * G + 15) & ~(size_t)15));
+  unsigned char *s_state = smem + warp_state_off(M, nv, nmom, TD);
   for (int i = threadIdx.x; i < M; i += blockDim.x) {
     s_c[i] = d.c[i];
     s_rd[i] = d.rdesc[i];
+    if (TD) s_beta[i] = d.beta[i];
   }
   for (int i = threadIdx.x; i < nv; i += blockDim.x) s_vl[i] = d.vlist[i];
   for (int i = threadIdx.x; i <= M; i += blockDim.x) s_vp[i] = d.vptr[i];
-  for (int i = threadIdx.x; i < M * G; i += blockDim.x) s_dep[i] = depg[i];
   for (int64_t i = threadIdx.x; i < nmom; i += blockDim.x) s_mom[i] = 0ull;
   __syncthreads();
-  const WarpNet net{M, N, nv, s_rd, s_c, s_vp, s_vl, s_dep};
+  const WarpNet net{M, N, s_rd, s_c, s_vp, TD ? d.vlist : s_vl, d.dptr, d.dlist, s_beta};
   const int warp = threadIdx.x >> 5;
   const int64_t j0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * S;
   if (j0 < A.n_traj)
-    warp_trajectories<R, G, LL>(A, net, s_X + warp * S * N, use_mom ? s_mom : nullptr, j0, tend_finite);
+    warp_trajectories<R, G, LL, TD>(A, net, s_state + (size_t)warp * S * warp_seg_bytes(M, N, G),
+                                    use_mom ? s_mom : nullptr, j0, tend_finite);
   if (use_mom) {
     __syncthreads();
     for (int64_t i = threadIdx.x; i < GN; i += blockDim.x) {
@@ -150,173 +161,6 @@ __device__ __forceinline__ void warp_write_outputs(const RunArgs &A, int64_t j, 
     if (A.out.status_dev) A.out.status_dev[j] = status;
     if (A.out.t_last_dev) A.out.t_last_dev[j] = t;
   }
-}
-
-// ---------------------------------------------------------------------------------
-// Time-dependent rates c_k(t) = c_k (1 + beta_k t) (Sec. 6, Eq. 29) for networks of up to
-// 256 reactions: a warp per trajectory, channel k in lane k % 32, register slot k / 32.
-// Every waiting time is the root of its channel's own integral, computed exactly (the
-// float-bound filter of the constant-rate routines is for plain quotients only); a warp
-// shuffle on (waiting time bits, channel) gives the smallest, smallest index on ties.  The
-// same operations, in the same order per channel, as the one-thread routine, so the results
-// are bit-identical to it and to the oracle.
-// ---------------------------------------------------------------------------------
-template <int R, bool LL>
-__global__ void __launch_bounds__(kWarpBlock) k_ens_tdep_warp(const RunArgs A, const int tend_finite) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  constexpr unsigned FULL = 0xFFFFFFFFu;
-  const DevNet &d = A.net;
-  const int M = d.M, N = d.N;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t j = (int64_t)blockIdx.x * (kWarpBlock / 32) + warp;
-  if (j >= A.n_traj) return;  // whole warps only; the kernel has no block-wide barrier
-  int *X = (int *)smem + (size_t)warp * N;
-  auto xat = [&](int sp) { return X[sp]; };
-  const uint64_t g = (uint64_t)(A.traj_offset + j);
-  const bool bad = warp_load_x0(A, j, X, lane);
-  double P[R], T[R], a[R], bt[R];
-  int32_t n[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int k = lane + 32 * r;
-    n[r] = 0;
-    T[r] = 0.0;
-    P[r] = 0.0;
-    a[r] = 0.0;
-    bt[r] = k < M ? d.beta[k] : 0.0;
-    if (!bad && k < M) {
-      P[r] = exp1_draw(A.seed, g, (uint32_t)k, 0u, A.stream_id);
-      a[r] = propensity(d.rdesc[k], d.c[k], xat);
-    }
-  }
-  int status = bad ? RT_TRAJ_BAD_X0 : RT_TRAJ_TEND;
-  double t = 0.0, ll = 0.0;
-  int32_t ev = 0;
-  int64_t gi = 0;
-  double next_g = 0.0;
-  auto record = [&](int64_t gidx, bool known) { warp_record(A, j, X, lane, gidx, known); };
-  if (!bad) {
-    const int64_t tend_bits = dbits(A.t_end);
-    for (;;) {
-      int64_t best = kInfBits;
-      int kb = INT_MAX;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int k = lane + 32 * r;
-        if (k < M && dbits(a[r]) != 0) {
-          const int64_t wb = dbits(tdep_wait(a[r], bt[r], __dsub_rn(P[r], T[r]), t));
-          if (wb < best) {
-            best = wb;
-            kb = k;
-          }
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const int64_t w2 = __shfl_xor_sync(FULL, best, o);
-        const int k2 = __shfl_xor_sync(FULL, kb, o);
-        if (w2 < best || (w2 == best && k2 < kb)) {
-          best = w2;
-          kb = k2;
-        }
-      }
-      if (kb == INT_MAX) {
-        status = RT_TRAJ_ABSORBED;
-        break;
-      }
-      const double dmin = bitsd(best);
-      const double tn = __dadd_rn(t, dmin);
-      if (dbits(tn) > tend_bits) {
-        status = RT_TRAJ_TEND;
-        break;
-      }
-      if (ev == A.max_events) {
-        status = RT_TRAJ_MAX_EVENTS;
-        break;
-      }
-      if (warp_overflow(d, kb, X, lane)) {
-        status = RT_TRAJ_OVERFLOW;
-        break;
-      }
-      while (gi < A.G && dbits(next_g) < dbits(tn)) {
-        record(gi, true);
-        ++gi;
-        next_g = __dmul_rn(__ll2double_rn(gi), A.sample_dt);
-      }
-      const double tprev = t;
-      t = tn;
-      if (lane == 0) trace_event(A.out, j, ev, kb, tn);
-      const int ol = kb & 31, os = kb >> 5;
-      const double a_mu = __shfl_sync(FULL, pick<R>(a, os), ol);
-      const double b_mu = __shfl_sync(FULL, pick<R>(bt, os), ol);
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        if (lane + 32 * r < M) T[r] = __dadd_rn(T[r], __dmul_rn(a[r], tdep_integral(bt[r], tprev, dmin)));
-      if (LL && lane == 0) ll = __dadd_rn(ll, rt_ln(__dmul_rn(a_mu, __dadd_rn(1.0, __dmul_rn(b_mu, t)))));
-      warp_fire(d, kb, X, lane);
-      if (lane == ol) {
-        int32_t nmu = 0;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-          if (r == os) {
-            n[r] += 1;
-            nmu = n[r];
-          }
-        const double E = exp1_draw(A.seed, g, (uint32_t)kb, (uint32_t)nmu, A.stream_id);
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-          if (r == os) P[r] = __dadd_rn(P[r], E);
-      }
-      ++ev;
-      const uint32_t dm = d.depw[(size_t)kb * 32 + lane];
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        if ((dm >> r) & 1u) a[r] = propensity(d.rdesc[lane + 32 * r], d.c[lane + 32 * r], xat);
-    }
-  }
-  const bool known = status == RT_TRAJ_TEND || status == RT_TRAJ_ABSORBED;
-  for (; gi < A.G; ++gi) record(gi, known);
-  if (A.out.loglik_dev || A.out.t_internal_dev) {
-    if (known && tend_finite && !bad) {
-      const double rest = __dsub_rn(A.t_end, t);
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        if (lane + 32 * r < M) T[r] = __dadd_rn(T[r], __dmul_rn(a[r], tdep_integral(bt[r], t, rest)));
-    }
-  }
-  warp_write_outputs<R>(A, j, X, lane, bad, T, n, ll, ev, status, t);
-}
-
-template <int R>
-static cudaError_t launch_tdep_r(const RunArgs &a, cudaStream_t s, int tend_finite) {
-  const size_t smem = (size_t)a.net.N * 4 * (kWarpBlock / 32);
-  const unsigned grid = (unsigned)((a.n_traj + kWarpBlock / 32 - 1) / (kWarpBlock / 32));
-  auto kern = a.out.loglik_dev ? k_ens_tdep_warp<R, true> : k_ens_tdep_warp<R, false>;
-  raise_smem_limit((const void *)kern, smem);
-  kern<<<grid, kWarpBlock, smem, s>>>(a, tend_finite);
-  return cudaGetLastError();
-}
-
-int launch_tdep_warp_mapping(const RunArgs &a, int lanes_per_traj, cudaStream_t s) {
-  if (a.n_traj == 0) return RT_OK;
-  const int M = a.net.M;
-  if (lanes_per_traj != 0 && lanes_per_traj != 32)
-    return set_error(RT_ERR_UNSUPPORTED, "time-dependent rates on the warp mapping use 32 lanes per trajectory");
-  if (M > 256 || !a.net.depw || !a.net.beta)
-    return set_error(RT_ERR_UNSUPPORTED, "time-dependent rates run on the warp mapping with M <= 256 (got %d)", M);
-  if ((size_t)a.net.N * 4 * (kWarpBlock / 32) > 200 * 1024)
-    return set_error(RT_ERR_UNSUPPORTED, "warp mapping: too many species for shared memory");
-  if ((a.n_traj + kWarpBlock / 32 - 1) / (kWarpBlock / 32) > INT_MAX)
-    return set_error(RT_ERR_UNSUPPORTED, "warp mapping: too many trajectories for one launch");
-  const int tf = std::isfinite(a.t_end) ? 1 : 0;
-  const int need = (M + 31) / 32;
-  cudaError_t e;
-  if (need <= 1) e = launch_tdep_r<1>(a, s, tf);
-  else if (need <= 2) e = launch_tdep_r<2>(a, s, tf);
-  else if (need <= 4) e = launch_tdep_r<4>(a, s, tf);
-  else e = launch_tdep_r<8>(a, s, tf);
-  if (e != cudaSuccess) return set_error(RT_ERR_CUDA, "time-dependent warp kernel launch: %s", cudaGetErrorString(e));
-  return RT_OK;
 }
 
 // ---------------------------------------------------------------------------------
@@ -496,27 +340,57 @@ int launch_rescaled_warp_mapping(const RunArgs &a, int lanes_per_traj, cudaStrea
 
 int warp_mapping_max_m() { return 256; }
 
-static size_t warp_net_bytes(const DevNet &d, int G) {
-  return (size_t)d.M * (8 + 8) + (size_t)d.n_vnz * 8 + (size_t)(d.M + 1) * 4 + (((size_t)d.M * G + 15) & ~(size_t)15);
-}
-
-template <int R, int G>
+template <int R, int G, bool TD>
 static cudaError_t launch_rg(const RunArgs &a, cudaStream_t s, int tend_finite) {
-  constexpr int wpb = kWarpBlock / 32, S = 32 / G;
-  const size_t mom = warp_moment_bytes(a);
-  const size_t smem = warp_net_bytes(a.net, G) + mom + (size_t)a.net.N * 4 * wpb * S;
+  constexpr int S = 32 / G;
+  const size_t per_warp = S * warp_seg_bytes(a.net.M, a.net.N, G);
+  const int nv = TD ? 0 : a.net.n_vnz;  // TD reads the net changes from global memory
+  size_t mom = warp_moment_bytes(a);
+  if (warp_state_off(a.net.M, nv, (int64_t)(mom / 8), TD) + per_warp > kWarpSmemMax) mom = 0;  // added in global memory
+  const size_t off = warp_state_off(a.net.M, nv, (int64_t)(mom / 8), TD);
+  int wpb = kWarpBlock / 32;  // fewer warps per block where many species or moments leave no room
+  while (wpb > 1 && off + wpb * per_warp > kWarpSmemMax) wpb /= 2;
+  const size_t smem = off + wpb * per_warp;
   const int64_t per_block = (int64_t)wpb * S;
+  if ((a.n_traj + per_block - 1) / per_block > INT_MAX) return cudaErrorInvalidConfiguration;
   const unsigned grid = (unsigned)((a.n_traj + per_block - 1) / per_block);
-  auto kern = a.out.loglik_dev ? k_ens_warp<R, G, true> : k_ens_warp<R, G, false>;
+  auto kern = a.out.loglik_dev ? k_ens_warp<R, G, true, TD> : k_ens_warp<R, G, false, TD>;
   raise_smem_limit((const void *)kern, smem);
-  kern<<<grid, kWarpBlock, smem, s>>>(a, tend_finite, mom ? 1 : 0);
+  kern<<<grid, wpb * 32, smem, s>>>(a, tend_finite, mom ? 1 : 0);
   return cudaGetLastError();
 }
 
-// Lanes per trajectory: 8 up to 64 reactions, 16 up to 128, else 32 (at most 8 channels per lane).
+template <bool TD>
+static cudaError_t launch_g(const RunArgs &a, int G, cudaStream_t s, int tf) {
+  const int need = (a.net.M + G - 1) / G;
+  if (G == 32) {
+    if (need <= 1) return launch_rg<1, 32, TD>(a, s, tf);
+    if (need <= 2) return launch_rg<2, 32, TD>(a, s, tf);
+    if (need <= 4) return launch_rg<4, 32, TD>(a, s, tf);
+    return launch_rg<8, 32, TD>(a, s, tf);
+  }
+  if (G == 16) {
+    if (need <= 4) return launch_rg<4, 16, TD>(a, s, tf);
+    return launch_rg<8, 16, TD>(a, s, tf);
+  }
+  if (need <= 2) return launch_rg<2, 8, TD>(a, s, tf);
+  if (need <= 4) return launch_rg<4, 8, TD>(a, s, tf);
+  return launch_rg<8, 8, TD>(a, s, tf);
+}
+
+// Lanes per trajectory: 8 up to 64 reactions, 16 up to 128, else 32: the fewest with at most eight
+// channels per lane, since the work of one event that is not per channel is shared by the warp's
+// trajectories (10000 trajectories, 8 / 16 / 32 lanes: M = 20 2.1 / 3.1 / 3.7 ms, M = 64 13.2 / 16.4 /
+// 21.7 ms, M = 100 - / 23.3 / 28.1 ms; sixteen channels per lane on 16 lanes lose at M = 256, 58 / 42 ms).
 static int choose_lanes(int M, int requested) {
   if (requested > 0) return requested;
   return M <= 64 ? 8 : M <= 128 ? 16 : 32;
+}
+
+// Shared memory one warp of a block needs, its block's tables included: what a network must fit in.
+static size_t warp_fit_bytes(const DevNet &d, int G) {
+  return (size_t)d.M * (8 + 8) + (size_t)d.n_vnz * 8 + (size_t)(d.M + 1) * 4 + (((size_t)d.M * G + 15) & ~(size_t)15) +
+         (size_t)d.N * 4 * (kWarpBlock / 32) * (32 / G);
 }
 
 int launch_warp_mapping(const RunArgs &a, int block_threads, int lanes_per_traj, cudaStream_t s) {
@@ -526,32 +400,34 @@ int launch_warp_mapping(const RunArgs &a, int block_threads, int lanes_per_traj,
   const int G = choose_lanes(M, lanes_per_traj);
   if (G != 8 && G != 16 && G != 32)
     return set_error(RT_ERR_INVALID_ARG, "warp mapping: lanes_per_traj must be 8, 16 or 32 (got %d)", G);
-  if (M > 8 * G) return set_error(RT_ERR_UNSUPPORTED, "warp mapping with %d lanes per trajectory supports M <= %d (got %d)",
-                                  G, 8 * G, M);
-  const uint8_t *dep = G == 8 ? a.net.depw8 : G == 16 ? a.net.depw16 : a.net.depw;
-  if (!dep) return set_error(RT_ERR_UNSUPPORTED, "warp mapping: no dependency table for %d lanes", G);
-  const size_t smem = warp_net_bytes(a.net, G) + (size_t)a.net.N * 4 * (kWarpBlock / 32) * (32 / G);
-  if (smem > 200 * 1024) return set_error(RT_ERR_UNSUPPORTED, "warp mapping: network too large for shared memory");
+  if (lanes_per_traj > 0 && M > 8 * G)
+    return set_error(RT_ERR_UNSUPPORTED, "warp mapping with %d lanes per trajectory supports M <= %d (got %d)", G, 8 * G, M);
+  if (M > 256) return set_error(RT_ERR_UNSUPPORTED, "warp mapping supports M <= 256 (got %d)", M);
+  if (warp_fit_bytes(a.net, G) > 200 * 1024)
+    return set_error(RT_ERR_UNSUPPORTED, "warp mapping: network too large for shared memory");
   const int64_t per_block = (int64_t)(kWarpBlock / 32) * (32 / G);
   if ((a.n_traj + per_block - 1) / per_block > INT_MAX)
     return set_error(RT_ERR_UNSUPPORTED, "warp mapping: too many trajectories for one launch");
-  const int tf = std::isfinite(a.t_end) ? 1 : 0;
-  const int need = (M + G - 1) / G;
-  cudaError_t e;
-  if (G == 32) {
-    if (need <= 1) e = launch_rg<1, 32>(a, s, tf);
-    else if (need <= 2) e = launch_rg<2, 32>(a, s, tf);
-    else if (need <= 4) e = launch_rg<4, 32>(a, s, tf);
-    else e = launch_rg<8, 32>(a, s, tf);
-  } else if (G == 16) {
-    if (need <= 4) e = launch_rg<4, 16>(a, s, tf);
-    else e = launch_rg<8, 16>(a, s, tf);
-  } else {
-    if (need <= 2) e = launch_rg<2, 8>(a, s, tf);
-    else if (need <= 4) e = launch_rg<4, 8>(a, s, tf);
-    else e = launch_rg<8, 8>(a, s, tf);
-  }
+  const cudaError_t e = launch_g<false>(a, G, s, std::isfinite(a.t_end) ? 1 : 0);
   if (e != cudaSuccess) return set_error(RT_ERR_CUDA, "warp kernel launch: %s", cudaGetErrorString(e));
+  return RT_OK;
+}
+
+int launch_tdep_warp_mapping(const RunArgs &a, int lanes_per_traj, cudaStream_t s) {
+  if (a.n_traj == 0) return RT_OK;
+  const int M = a.net.M;
+  if (lanes_per_traj != 0 && lanes_per_traj != 32)
+    return set_error(RT_ERR_UNSUPPORTED, "time-dependent rates on the warp mapping use 32 lanes per trajectory");
+  if (M > 256 || !a.net.beta)
+    return set_error(RT_ERR_UNSUPPORTED, "time-dependent rates run on the warp mapping with M <= 256 (got %d)", M);
+  if ((size_t)a.net.N * 4 * (kWarpBlock / 32) > 200 * 1024)
+    return set_error(RT_ERR_UNSUPPORTED, "warp mapping: too many species for shared memory");
+  if ((a.n_traj + kWarpBlock / 32 - 1) / (kWarpBlock / 32) > INT_MAX)
+    return set_error(RT_ERR_UNSUPPORTED, "warp mapping: too many trajectories for one launch");
+  int G = choose_lanes(M, lanes_per_traj);
+  if (warp_state_off(M, 0, 0, true) + (32 / G) * warp_seg_bytes(M, a.net.N, G) > kWarpSmemMax) G = 32;  // many species
+  const cudaError_t e = launch_g<true>(a, G, s, std::isfinite(a.t_end) ? 1 : 0);
+  if (e != cudaSuccess) return set_error(RT_ERR_CUDA, "time-dependent warp kernel launch: %s", cudaGetErrorString(e));
   return RT_OK;
 }
 
