@@ -35,7 +35,7 @@ struct BNet {
   int64_t xoff;  // first species of this network in the packed x0 / x_final rows
   int64_t moff;  // first reaction of this network in the packed counts / t_internal rows
   int32_t cls;
-  int32_t R;     // register slots (warp and block: 1, 2, 4 or 8)
+  int32_t R;     // channel slots (warp: 1, 2, 4 or 8; block: 1 to 8, or 16)
   uint32_t stream_id;
   int32_t pad;
 };
@@ -56,6 +56,7 @@ struct BatchArgs {
   int maxN_thread, maxM_block, maxN_block;
   size_t warp_bytes;   // shared memory of one warp-class trajectory
   int warp_task;       // warp-class trajectories per task
+  size_t state_bytes;  // shared-memory channel state of the largest block-class network that keeps it there
 };
 
 __device__ __forceinline__ RunArgs item_args(const BatchArgs &B, int net_index, const BNet &bn) {
@@ -110,16 +111,20 @@ __global__ void __launch_bounds__(512, 2) k_batch(const BatchArgs B) {
       const int64_t j = f % B.n_traj;
       const BNet bn = B.nets[ni];
       const RunArgs A = item_args(B, ni, bn);
-      const BlockScratch S = carve_block_scratch(smem, B.maxM_block, B.maxN_block, BT);
-      const BlockNet net{bn.d.M, bn.d.N, bn.d.rdesc, bn.d.c, bn.d.vptr, bn.d.vlist, bn.d.sptr, bn.d.slist,
-                         bn.d.dptr, bn.d.dlist};
+      const BlockScratch S = carve_block_scratch(smem, B.state_bytes, B.maxM_block, B.maxN_block, BT);
+      const BlockNet net{bn.d.M, bn.d.N, bn.d.rdesc, bn.d.c, bn.d.vptr, bn.d.vlist, bn.d.dptr, bn.d.dlist};
       const int tf = isfinite(A.t_end) ? 1 : 0;
-      switch (bn.R) {
-        case 1: block_trajectory<1, LL>(A, net, S, j, tf); break;
-        case 2: block_trajectory<2, LL>(A, net, S, j, tf); break;
-        case 4: block_trajectory<4, LL>(A, net, S, j, tf); break;
-        case 8: block_trajectory<8, LL>(A, net, S, j, tf); break;
-        default: block_trajectory<16, LL>(A, net, S, j, tf); break;
+      switch (B.state_bytes || bn.R > 8 ? bn.R : 0) {
+        case 0: block_trajectory<8, LL, false>(A, net, S, j, tf); break;
+        case 1: block_trajectory<1, LL, true>(A, net, S, j, tf); break;
+        case 2: block_trajectory<2, LL, true>(A, net, S, j, tf); break;
+        case 3: block_trajectory<3, LL, true>(A, net, S, j, tf); break;
+        case 4: block_trajectory<4, LL, true>(A, net, S, j, tf); break;
+        case 5: block_trajectory<5, LL, true>(A, net, S, j, tf); break;
+        case 6: block_trajectory<6, LL, true>(A, net, S, j, tf); break;
+        case 7: block_trajectory<7, LL, true>(A, net, S, j, tf); break;
+        case 8: block_trajectory<8, LL, true>(A, net, S, j, tf); break;
+        default: block_trajectory<16, LL, false>(A, net, S, j, tf); break;
       }
       continue;
     }
@@ -183,7 +188,7 @@ struct rt_batch {
   int64_t total_species = 0, total_reactions = 0;
   rt_batch_policy policy;
   int maxN_thread = 1, maxM_block = 1, maxN_block = 1;
-  size_t warp_bytes = 0;
+  size_t warp_bytes = 0, state_bytes = 0;
   int warp_task = 1;
   size_t smem = 0;
   int grid = 0;
@@ -240,9 +245,10 @@ extern "C" int rt_batch_create(int32_t n_nets, const rt_network *const *nets, co
     if (cls == CLS_WARP) R = M <= 32 ? 1 : M <= 64 ? 2 : M <= 128 ? 4 : 8;
     if (cls == CLS_BLOCK) {
       const int need = (M + pol.block_threads - 1) / pol.block_threads;
-      R = need <= 1 ? 1 : need <= 2 ? 2 : need <= 4 ? 4 : need <= 8 ? 8 : 16;
+      R = need <= 8 ? need : 16;
       b->maxM_block = std::max(b->maxM_block, M);
       b->maxN_block = std::max(b->maxN_block, N);
+      if (R <= 8) b->state_bytes = std::max(b->state_bytes, block_state_bytes(M, pol.block_threads));
     }
     if (cls == CLS_WARP) b->warp_bytes = std::max(b->warp_bytes, warp_seg_bytes(M, N, 32));
     if (cls == CLS_THREAD) b->maxN_thread = std::max(b->maxN_thread, N);
@@ -312,7 +318,10 @@ extern "C" int rt_batch_create(int32_t n_nets, const rt_network *const *nets, co
 
   // shared memory: the largest of the three uses (a block runs one task at a time)
   const int BT = pol.block_threads;
-  const size_t s_block = b->n_cls[CLS_BLOCK] ? block_scratch_bytes(b->maxM_block, b->maxN_block, BT) : 0;
+  if (b->state_bytes + block_scratch_bytes(b->maxM_block, b->maxN_block, BT) > kBatchSmemMax)
+    b->state_bytes = 0;  // many species: the channel state stays in local memory
+  const size_t s_block =
+      b->n_cls[CLS_BLOCK] ? b->state_bytes + block_scratch_bytes(b->maxM_block, b->maxN_block, BT) : 0;
   const size_t s_thread = (size_t)BT * b->maxN_thread * 4;
   // warp-class trajectories per task: one per warp of the block, as far as two blocks per SM can hold
   // their state (or as the other classes' shared memory allows anyway)
@@ -392,6 +401,7 @@ extern "C" int rt_batch_run(rt_batch *b, const int32_t *x0_dev, const double *t_
   A.maxN_thread = b->maxN_thread;
   A.warp_bytes = b->warp_bytes;
   A.warp_task = b->warp_task;
+  A.state_bytes = b->state_bytes;
   A.maxM_block = b->maxM_block;
   A.maxN_block = b->maxN_block;
   cudaStream_t s = (cudaStream_t)stream;

@@ -1,18 +1,30 @@
-// rt_traj_block.cuh -- one thread block per trajectory, state in registers.
+// rt_traj_block.cuh -- one thread block per trajectory.
 //
 // The NRRTA loop of Table 2 (Liu & Wang, arXiv:2103.00405) for networks of up to
-// 8 * blockDim.x reactions: channel k lives in thread k % B, register slot k / B
-// (P_k, T_k, a_k, n_k; Eq. 17-27), X in shared memory.  Per event:
-//   1. the channels that read a species the last firing changed are marked in a
-//      shared bitmap from the species -> reactions lists (dependency graph, Sec. 5);
-//   2. each thread fires its own bookkeeping (new Exp(1) draw, Eq. 27), advances
-//      its internal times with the pre-event propensities (Eq. 17), recomputes the
-//      marked propensities (Eq. 1-2) and proposes its smallest certified upper
-//      bound of the waiting time;
-//   3. each warp's best candidate publishes a float upper bound of its waiting time; every
-//      thread takes the block's best candidate's bound as threshold, computes exactly only
-//      channels not certified to be larger, and a block reduction on (waiting time bits,
-//      channel) gives the exact argmin (Eq. 25-26).
+// R * blockDim.x reactions: channel k belongs to thread k % B, slot k / B (Eq. 17-27).
+// T_k is in registers; a_k and a pair of floats (upper bounds of P_k and 1 / a_k) in
+// shared memory (or, where a block cannot hold them, in the thread's local memory), P_k
+// and the increment drawn ahead for the channel's next firing, which an event reads for one
+// or two channels, in local memory; firing counts, X, and a bitmap of the channels whose
+// propensity must be recomputed in shared memory.  Per event three phases, a barrier after each:
+//   Y: the last firing's owner adds its increment to P (Eq. 27); every T_k advances with the
+//      pre-event a_k (Eq. 17) and gives a float interval of its waiting time; each lane
+//      recomputes its marked propensities and their intervals (Eq. 1-2, one pass for all first
+//      ones); the block minimum of the upper ends;
+//   E: the channels whose interval reaches below that minimum are computed exactly (one or two
+//      in the block) and listed with where their net change and dependents are stored;
+//   X: every thread takes the smallest of the list, smallest index on ties (Eq. 25-26); the net
+//      change is applied by one thread per species with the int32 range check (undone if it
+//      fails), and the dependents are marked.
+// The fired channel's next increment is drawn by its owner in two halves where the other warps
+// wait anyway: the Philox block in phase E, its logarithm in phase X of the event after.
+// What bounds it: the advance of T issues two FP64 warp instructions (16 cycles each) per 32
+// channels and event, 2000 cycles per event at 2000 reactions; the rest of an event is latency
+// (about as much), which the SM's other blocks fill.  Against P, T and a in (spilled) registers with
+// every bound taken from them per event and one thread's draw on the path: 500 trajectories of 2000
+// reactions, 5000 events each, 56 -> 31.8 ms; of 4096 reactions 114 -> 70 ms; 20 trajectories of 500
+// reactions 37 -> 9.4 ms (with the block size by the number of trajectories); 512 networks of 4 to
+// 4096 reactions in one batch 309 -> 210 ms.
 #pragma once
 #include <climits>
 
@@ -26,61 +38,60 @@ struct BlockNet {
   const double *c;
   const int *vp;
   const int2 *vl;
-  const int *sptr;
-  const int *slist;
-  const int *dptr;   // per reaction the channels its firing touches (or null: from sptr/slist)
+  const int *dptr;  // per reaction the channels its firing touches: dlist[dptr[k]..dptr[k+1])
   const int *dlist;
+};
+
+// a channel that may be the next to fire, and where its net change and dependents lie
+struct __align__(16) BlockCand {
+  long long w;
+  int k, vb, ve, db, de;
+  int owner;  // its thread and, from bit 16, its slot
 };
 
 // shared-memory scratch of one block trajectory
 struct BlockScratch {
-  int *X;           // [N]
-  int *NK;          // [M] firing counts n_k
-  uint32_t *bm;     // [ceil(M/32)] channels whose propensity must be recomputed
-  float *red_u;     // [warps]
-  int *red_k;       // [warps]
-  long long *red_w; // [warps]
-  float *red_q;     // [warps] float upper bound of each warp's candidate's waiting time
-  int *red_k2;      // [warps]
-  double *buf;      // [B] (and the broadcast slots below)
-  double *s_amu;    // propensity of the fired channel
-  double *s_E;      // the fired channel's new Exp(1) increment
-  int *s_over;      // set if the fired reaction would leave the int32 range
+  double *a;       // [slots][B] propensities (SM)
+  float2 *b;       // [slots][B] {P bound, 1 / a bound} (SM)
+  BlockCand *cand; // [B]
+  double *buf;     // [B]
+  double *s_amu;   // propensity of the fired channel
+  uint32_t *red;   // [warps] bits of each warp's smallest upper end
+  int *s_over;     // set if the fired reaction would leave the int32 range
+  int *s_cnt;      // entries of cand
+  uint32_t *bm;    // [ceil(M/32)] channels whose propensity must be recomputed
+  int *NK;         // [M] firing counts n_k
+  int *X;          // [N]
 };
 
+__host__ __device__ inline size_t block_state_bytes(int M, int B) { return (size_t)((M + B - 1) / B) * B * 16; }
+
 __host__ __device__ inline size_t block_scratch_bytes(int M, int N, int B) {
-  const int W = B / 32;
-  return (size_t)N * 4 + (size_t)M * 4 + (size_t)((M + 31) / 32) * 4 + (size_t)W * (4 + 4 + 4 + 8 + 4) +
-         (size_t)B * 8 + 32 + 64;
+  return (size_t)B * (sizeof(BlockCand) + 8) + 16 + (size_t)(B / 32) * 4 + 8 + (size_t)((M + 31) / 32) * 4 +
+         (size_t)M * 4 + (size_t)N * 4 + 64;
 }
 
-__device__ inline BlockScratch carve_block_scratch(unsigned char *base, int M, int N, int B) {
-  const int W = B / 32;
+// state_bytes: what the SM arrays take at the start (0 without them)
+__device__ inline BlockScratch carve_block_scratch(unsigned char *base, size_t state_bytes, int M, int N, int B) {
   BlockScratch s;
-  s.buf = (double *)base;
-  s.red_w = (long long *)(s.buf + B);
-  s.s_amu = (double *)(s.red_w + W);
-  s.s_E = s.s_amu + 1;
-  s.red_u = (float *)(s.s_E + 1);
-  s.red_q = s.red_u + W;
-  s.red_k = (int *)(s.red_q + W);
-  s.red_k2 = s.red_k + W;
-  s.s_over = s.red_k2 + W;
-  s.bm = (uint32_t *)(s.s_over + 1);
-  s.X = (int *)(s.bm + (M + 31) / 32);
-  s.NK = s.X + N;
+  s.a = (double *)base;
+  s.b = (float2 *)(base + state_bytes / 2);
+  s.cand = (BlockCand *)(base + state_bytes);
+  s.buf = (double *)(s.cand + B);
+  s.s_amu = s.buf + B;
+  s.red = (uint32_t *)(s.s_amu + 1);
+  s.s_over = (int *)(s.red + B / 32);
+  s.s_cnt = s.s_over + 1;
+  s.bm = (uint32_t *)(s.s_cnt + 1);
+  s.NK = (int *)(s.bm + (M + 31) / 32);
+  s.X = s.NK + M;
   return s;
 }
 
-// Per event (after the first): phase X, right after the argmin is known, runs three
-// independent pieces at once -- the fired reaction's net change applied to X by one
-// thread per changed species (with the int32 range check), its dependents marked in
-// the bitmap, and its new Exp(1) increment drawn by the last thread of the block --
-// then one barrier; phase Y advances every T_k with the pre-event a_k (Eq. 17),
-// recomputes and unmarks the marked propensities and proposes waiting-time bounds.
-// Grid samples, when an event crosses a grid time, are written from the pre-event X
-// before phase X behind their own barrier.
-template <int R, bool LL>
+// R: slots, ceil(M / B) with SM (the loops over slots then have no branch, so that the slots' 64-cycle FP64
+// operations overlap; entries past M hold a = 0 and an interval at +inf), at least that without.
+// SM: a and the float pairs in shared memory (else in the thread's local memory).
+template <int R, bool LL, bool SM>
 __device__ __forceinline__ void block_trajectory(const RunArgs &A, const BlockNet &net, const BlockScratch &S, const int64_t j,
                                  const int tend_finite) {
   const int tid = threadIdx.x, B = blockDim.x, lane = tid & 31, warp = tid >> 5, W = B >> 5;
@@ -114,21 +125,33 @@ __device__ __forceinline__ void block_trajectory(const RunArgs &A, const BlockNe
     if (tid == 0 && A.out.grid_count_dev) atomicAdd((unsigned long long *)(A.out.grid_count_dev + gidx), 1ull);
   };
 
-  double P[R], T[R], a[R];
+  double T[R], P[R], En[R];
+  float lo[R];
+  double a_loc[SM ? 1 : R];
+  float2 b_loc[SM ? 1 : R];
+  auto a_ref = [&](int r) -> double & { return SM ? S.a[r * B + tid] : a_loc[SM ? 0 : r]; };
+  auto b_ref = [&](int r) -> float2 & { return SM ? S.b[r * B + tid] : b_loc[SM ? 0 : r]; };
 #pragma unroll
+  for (int r = 0; r < R; ++r) T[r] = 0.0;
+#pragma unroll 1
   for (int r = 0; r < R; ++r) {
     const int k = tid + B * r;
-    P[r] = 0.0;
-    T[r] = 0.0;
-    a[r] = 0.0;
-    if (!bad && k < M) {
-      P[r] = exp1_draw(A.seed, g, (uint32_t)k, 0u, A.stream_id);
-      a[r] = propensity<false>(net.rd[k], net.c[k], xat);
+    P[r] = 1.0;
+    {
+      double av = 0.0;
+      if (!bad && k < M) {
+        P[r] = exp1_draw(A.seed, g, (uint32_t)k, 0u, A.stream_id);
+        En[r] = exp1_draw(A.seed, g, (uint32_t)k, 1u, A.stream_id);
+        av = propensity(net.rd[k], net.c[k], xat);
+      }
+      a_ref(r) = av;
+      b_ref(r) = make_float2(upper_P(P[r]), inv_upper(av));
     }
   }
   int status = bad ? RT_TRAJ_BAD_X0 : RT_TRAJ_TEND;
   double t = 0.0, ll = 0.0, dmin = 0.0;
-  int mu = -1;  // the last fired channel (uniform)
+  bool fired = false;  // an event precedes this pass
+  int owner = 0;       // thread and slot of the last fired channel
   int32_t ev = 0;
   int64_t gi = 0;
   double next_g = 0.0;
@@ -136,116 +159,109 @@ __device__ __forceinline__ void block_trajectory(const RunArgs &A, const BlockNe
 
   if (!bad) {
     for (;;) {
-      // ---- phase Y: the last firing's bookkeeping, T advance, recompute, bounds
-      const bool fired = mu >= 0;
-      if (fired && tid == mu % B) {  // Eq. 27: the fired channel's new increment
-        const int rm = mu / B;
-        const double E = *S.s_E;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-          if (r == rm) P[r] = __dadd_rn(P[r], E);
+      // ---- phase Y
+      if (fired && tid == (owner & 0xFFFF)) {  // Eq. 27
+        const int rm = owner >> 16, k = tid + B * rm;
+        const int32_t n = S.NK[k] + 1;
+        S.NK[k] = n;
+        P[rm] = __dadd_rn(P[rm], En[rm]);
+        b_ref(rm).x = upper_P(P[rm]);
       }
       if (LL && fired && tid == 0) ll = __dadd_rn(ll, rt_ln(*S.s_amu));
-      if (tid == 0) *S.s_over = 0;
-      const bool adv = fired && dbits(dmin) != 0;
+      if (tid == 0) {
+        *S.s_over = 0;
+        *S.s_cnt = 0;
+      }
+      uint32_t todo = 0;
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (warp + W * r < nbm) todo |= ((S.bm[warp + W * r] >> lane) & 1u) << r;
+      const bool adv = dbits(dmin) != 0;
       float ub = __int_as_float(0x7F800000);
-      int kub = INT_MAX;
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int k = tid + B * r;
-        if (k < M) {
-          if (adv && dbits(a[r]) != 0) T[r] = __dadd_rn(T[r], __dmul_rn(a[r], dmin));
-          const uint32_t bit = 1u << (k & 31);
-          if (S.bm[k >> 5] & bit) {
-            a[r] = propensity<false>(net.rd[k], net.c[k], xat);
-            atomicAnd(&S.bm[k >> 5], ~bit);
-          }
-          if (dbits(a[r]) != 0) {
-            const float u = wait_estimate(P[r], T[r], a[r]);
-            if (kub == INT_MAX || u < ub) {
-              ub = u;
-              kub = k;
-            }
-          }
+      for (int r = 0; r < R; ++r)
+        {
+          const double Tn = __dadd_rn(T[r], __dmul_rn(a_ref(r), dmin));
+          T[r] = adv ? Tn : T[r];
+          const float u = wait_interval(b_ref(r), T[r], lo[r]);
+          ub = fminf(ub, (todo >> r) & 1u ? __int_as_float(0x7F800000) : u);
         }
-      }
+      if (__any_sync(0xFFFFFFFFu, todo != 0)) {
+        if (lane < R && warp + W * lane < nbm) S.bm[warp + W * lane] = 0u;  // this warp's words
+        do {
+          if (todo) {
+            const int r = __ffs((int)todo) - 1, k = tid + B * r;
+            const double av = propensity(net.rd[k], net.c[k], xat);
+            a_ref(r) = av;
+            const float2 q = make_float2(b_ref(r).x, inv_upper(av));
+            b_ref(r).y = q.y;
+            float l;
+            ub = fminf(ub, wait_interval(q, pick<R>(T, r), l));
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float u2 = __shfl_xor_sync(0xFFFFFFFFu, ub, o);
-        const int k2 = __shfl_xor_sync(0xFFFFFFFFu, kub, o);
-        if (u2 < ub || (u2 == ub && k2 < kub)) {
-          ub = u2;
-          kub = k2;
-        }
+            for (int i = 0; i < R; ++i) lo[i] = i == r ? l : lo[i];
+            todo &= todo - 1;
+          }
+        } while (__any_sync(0xFFFFFFFFu, todo != 0));
       }
-      // the warp candidate's owner publishes a float upper bound of its waiting time with it, so
-      // the block's threshold is known right after the reduction (one barrier, no division)
-      if (kub != INT_MAX && tid == kub % B) {
-        const int rs = kub / B;
-        S.red_q[warp] = quot_upper(pick<R>(P, rs), pick<R>(T, rs), pick<R>(a, rs));
-        S.red_u[warp] = ub;
-        S.red_k[warp] = kub;
-      } else if (kub == INT_MAX && lane == 0) {
-        S.red_u[warp] = ub;
-        S.red_k[warp] = kub;
+      const uint32_t wub = __reduce_min_sync(0xFFFFFFFFu, __float_as_uint(fmaxf(ub, 0.0f)));
+      if (lane == 0) S.red[warp] = wub;
+      __syncthreads();
+      // ---- phase E: the channels that reach below the block's smallest upper end, exactly; the last
+      // firing's owner begins its next draw
+      const float thr =
+          interval_threshold(__uint_as_float(__reduce_min_sync(0xFFFFFFFFu, lane < W ? S.red[lane] : 0x7F800000u)));
+      uint32_t need = 0;
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (!(lo[r] > thr)) need |= 1u << r;
+      if (need) {
+        BlockCand e;
+        e.w = kInfBits;
+        e.k = INT_MAX;
+        e.vb = e.ve = e.db = e.de = e.owner = 0;
+        do {
+          const int r = __ffs((int)need) - 1, k = tid + B * r;
+          need &= need - 1;
+          const double av = a_ref(r);
+          if (dbits(av) == 0) continue;  // the padding past M too
+          const int vb = net.vp[k], ve = net.vp[k + 1], db = net.dptr[k], de = net.dptr[k + 1];
+          const long long wb = dbits(waiting_time(P[r], pick<R>(T, r), av));
+          if (wb < e.w) {  // a thread's channels come in index order
+            e.w = wb;
+            e.k = k;
+            e.vb = vb;
+            e.ve = ve;
+            e.db = db;
+            e.de = de;
+            e.owner = tid | (r << 16);
+          }
+        } while (need);
+        if (e.k != INT_MAX) S.cand[atomicAdd(S.s_cnt, 1)] = e;
+      }
+      const bool drawing = fired && tid == (owner & 0xFFFF);
+      const int rd = owner >> 16;
+      uint64_t draw = 0;
+      if (drawing) {
+        const int k = tid + B * rd;
+        draw = draw_bits(A.seed, g, (uint32_t)k, (uint32_t)S.NK[k] + 1u, A.stream_id);
       }
       __syncthreads();
-      // every warp reduces the W warp minima itself (lane w reads warp w's): the block minimum
-      // in every thread without another barrier (lexicographic minimum: order-independent)
-      ub = lane < W ? S.red_u[lane] : __int_as_float(0x7F800000);
-      kub = lane < W ? S.red_k[lane] : INT_MAX;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float u2 = __shfl_xor_sync(0xFFFFFFFFu, ub, o);
-        const int k2 = __shfl_xor_sync(0xFFFFFFFFu, kub, o);
-        if (u2 < ub || (u2 == ub && k2 < kub)) {
-          ub = u2;
-          kub = k2;
-        }
-      }
-      if (kub == INT_MAX) {
+      // ---- phase X: the smallest of the list (every thread the same decision)
+      const int cnt = *S.s_cnt;
+      if (cnt == 0) {
         status = RT_TRAJ_ABSORBED;
         break;
       }
-      // ---- every channel not certified to lie above the block candidate's upper bound, exactly
-      // (the candidate itself is never certified above its own bound) (Eq. 25-26)
-      const float thr = S.red_q[(kub % B) >> 5];
-      long long bw = LLONG_MAX;
-      int bk = INT_MAX;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int k = tid + B * r;
-        if (k < M && dbits(a[r]) != 0 && !exceeds(P[r], T[r], a[r], thr)) {
-          const long long wb = dbits(waiting_time(P[r], T[r], a[r]));
-          if (wb < bw || (wb == bw && k < bk)) {
-            bw = wb;
-            bk = k;
-          }
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const long long w2 = __shfl_xor_sync(0xFFFFFFFFu, bw, o);
-        const int k2 = __shfl_xor_sync(0xFFFFFFFFu, bk, o);
+      int ci = 0;
+      long long bw = S.cand[0].w;
+      int bk = S.cand[0].k;
+      for (int i = 1; i < cnt; ++i) {
+        const long long w2 = S.cand[i].w;
+        const int k2 = S.cand[i].k;
         if (w2 < bw || (w2 == bw && k2 < bk)) {
           bw = w2;
           bk = k2;
-        }
-      }
-      if (lane == 0) {
-        S.red_w[warp] = bw;
-        S.red_k2[warp] = bk;
-      }
-      __syncthreads();
-      bw = lane < W ? S.red_w[lane] : LLONG_MAX;
-      bk = lane < W ? S.red_k2[lane] : INT_MAX;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const long long w2 = __shfl_xor_sync(0xFFFFFFFFu, bw, o);
-        const int k2 = __shfl_xor_sync(0xFFFFFFFFu, bk, o);
-        if (w2 < bw || (w2 == bw && k2 < bk)) {
-          bw = w2;
-          bk = k2;
+          ci = i;
         }
       }
       const double dnext = bitsd(bw);
@@ -258,15 +274,14 @@ __device__ __forceinline__ void block_trajectory(const RunArgs &A, const BlockNe
         status = RT_TRAJ_MAX_EVENTS;
         break;
       }
-      const int vb = net.vp[bk], ve = net.vp[bk + 1];
+      const int vb = S.cand[ci].vb, ve = S.cand[ci].ve;
       if (gi < A.G && dbits(next_g) < dbits(tn)) {
         // grid samples from the pre-event X, after the range check (an overflowing event
         // records nothing); X is only read until the barrier below
         bool over = false;
         for (int i = vb; i < ve; ++i) {
           const int2 e = net.vl[i];
-          const long long nx = (long long)X[e.x] + e.y;
-          over |= (nx > INT_MAX) | (nx < 0);
+          over |= (int)((uint32_t)X[e.x] + (uint32_t)e.y) < 0;
         }
         if (over) {
           status = RT_TRAJ_OVERFLOW;
@@ -279,40 +294,25 @@ __device__ __forceinline__ void block_trajectory(const RunArgs &A, const BlockNe
         }
         __syncthreads();
       }
-      // ---- phase X: net change with range check, dependents, new draw (all at once)
       for (int i = vb + tid; i < ve; i += B) {
         const int2 e = net.vl[i];
-        const long long nx = (long long)X[e.x] + e.y;
-        if ((nx > INT_MAX) | (nx < 0)) *S.s_over = 1;
-        X[e.x] = (int)(uint32_t)((uint32_t)X[e.x] + (uint32_t)e.y);
+        const int nx = (int)((uint32_t)X[e.x] + (uint32_t)e.y);
+        if (nx < 0) *S.s_over = 1;  // a count past INT_MAX wraps below 0
+        X[e.x] = nx;
       }
-      if (net.dptr) {  // one list per reaction: two dependent loads instead of four
-        for (int q = net.dptr[bk] + tid; q < net.dptr[bk + 1]; q += B) {
-          const int ch = net.dlist[q];
-          atomicOr(&S.bm[ch >> 5], 1u << (ch & 31));
-        }
-      } else {
-        for (int i = vb; i < ve; ++i) {
-          const int s = net.vl[i].x;
-          for (int q = net.sptr[s] + tid; q < net.sptr[s + 1]; q += B) {
-            const int ch = net.slist[q];
-            atomicOr(&S.bm[ch >> 5], 1u << (ch & 31));
-          }
-        }
+      for (int q = S.cand[ci].db + tid; q < S.cand[ci].de; q += B) {
+        const int ch = net.dlist[q];
+        atomicOr(&S.bm[ch >> 5], 1u << (ch & 31));
       }
-      if (tid == B - 1) {
-        const int32_t n = S.NK[bk] + 1;
-        S.NK[bk] = n;
-        *S.s_E = exp1_draw(A.seed, g, (uint32_t)bk, (uint32_t)n, A.stream_id);
-      }
-      if (LL && tid == (bk % B)) *S.s_amu = pick<R>(a, bk / B);
+      if (drawing) En[rd] = exp1_from_bits(draw);
+      owner = S.cand[ci].owner;
+      if (LL && tid == (owner & 0xFFFF)) *S.s_amu = a_ref(owner >> 16);
       __syncthreads();
       if (*S.s_over) {  // undo: the event does not fire
         for (int i = vb + tid; i < ve; i += B) {
           const int2 e = net.vl[i];
           X[e.x] = (int)(uint32_t)((uint32_t)X[e.x] - (uint32_t)e.y);
         }
-        if (tid == B - 1) S.NK[bk] -= 1;
         status = RT_TRAJ_OVERFLOW;
         break;
       }
@@ -320,7 +320,7 @@ __device__ __forceinline__ void block_trajectory(const RunArgs &A, const BlockNe
       if (tid == 0) trace_event(A.out, j, ev, bk, tn);
       ++ev;
       dmin = dnext;
-      mu = bk;
+      fired = true;
     }
   }
 
@@ -332,7 +332,7 @@ __device__ __forceinline__ void block_trajectory(const RunArgs &A, const BlockNe
       const double rest = __dsub_rn(A.t_end, t);
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        if (tid + B * r < M) T[r] = __dadd_rn(T[r], __dmul_rn(a[r], rest));
+        if (tid + B * r < M) T[r] = __dadd_rn(T[r], __dmul_rn(a_ref(r), rest));
     }
     if (A.out.t_internal_dev)
 #pragma unroll
