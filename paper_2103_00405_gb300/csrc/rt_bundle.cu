@@ -18,6 +18,18 @@
 // K / sum(a) that catches all but ~e^-K of minima (sum(a) retaken every 64 events).
 // If no channel beat the threshold, the event is re-scanned without it (read-only),
 // so the minimum is always the exact one, with the smallest index on ties.
+//
+// P is kept as two arrays of words: the bounds read the high ones only, so the pass streams 28 bytes
+// per channel and event (T and a, the high word of P; T written back) instead of 32.  What bounds it
+// at 16 trajectories of 10^6 channels (144 blocks): the FP64 pipe 54 us of an event's 79 us (two
+// instructions per channel), memory 66 us at the copy rate, and about 10 us between passes; for one
+// trajectory or a few thousand channels only the time between passes matters.  That is a chain of
+// memory trips: the C minima are read by a warp in one trip, the barrier is polled without sleeping,
+// the fired reaction's record (prefetched by the block whose candidate it is) gives its net change and
+// reader lists in one trip, marks are cleared without reading the lists again, and the fired channel's
+// increment is drawn by the thread that scans it while the others begin.  500 events: 16 trajectories
+// of 10^6 reactions 43.6 -> 39.7 ms, one 12.6 -> 5.6 ms, 4 of 200000 7.6 -> 4.9 ms, one of 5000
+// 10.2 -> 3.7 ms.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -35,6 +47,7 @@ constexpr int kBundleThreads = 512;
 constexpr float kThresholdK = 12.0f;  // per-event threshold K / sum(a): P(re-scan) ~ e^-12
 constexpr int kSumEvery = 64;         // events between two sums of a (the threshold's sum(a))
 constexpr int kMaxDepth = 6;          // stages of the per-thread copy ring, at most
+constexpr size_t kStageBytes = (size_t)kBundleThreads * (16 + 16 + 8);
 
 struct __align__(16) Partial {
   long long wbits;  // bits of the block's minimum waiting time (+inf if none)
@@ -51,7 +64,8 @@ struct BundleArgs {
   int64_t traj0;     // first trajectory of this launch
   int64_t Ms;        // row stride of P/T/A/NK (multiple of 32)
   int64_t chunk;     // channels per block slice (multiple of 32)
-  double *P, *T, *A;
+  uint32_t *Ph, *Pl;  // high and low words of P: the scan streams the high ones
+  double *T, *A;
   int32_t *NK;
   Partial *part;     // [n_traj][2][C]
   unsigned long long *bar;  // [n_traj] monotonic arrival counters
@@ -75,7 +89,7 @@ __device__ bool bundle_barrier(unsigned long long *ctr, unsigned long long targe
   long long it = 0;
   while (ld_acquire(ctr) < target) {
     if (++it > limit) return false;
-    __nanosleep(100);
+    if (it > 256) __nanosleep(100);  // a sleep lasts about a microsecond, a poll a third of one
   }
   __threadfence();
   return true;
@@ -91,7 +105,9 @@ __global__ void k_bundle_init(const BundleArgs B) {
     const int64_t o = j * B.Ms + k;
     B.T[o] = 0.0;
     B.NK[o] = 0;
-    B.P[o] = exp1_draw(r.seed, (uint64_t)(r.traj_offset + j), (uint32_t)k, 0u, r.stream_id);
+    const double P = exp1_draw(r.seed, (uint64_t)(r.traj_offset + j), (uint32_t)k, 0u, r.stream_id);
+    B.Ph[o] = (uint32_t)__double2hiint(P);
+    B.Pl[o] = (uint32_t)__double2loint(P);
     B.A[o] = propensity<false>(r.net.rdesc[k], r.net.c[k], [&](int s) { return x0[s]; });
   }
 }
@@ -99,6 +115,10 @@ __global__ void k_bundle_init(const BundleArgs B) {
 // ---- per-thread asynchronous global -> shared copies (16 B) in commit groups ----
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
@@ -125,13 +145,14 @@ struct Decision {
 };
 
 template <bool LL>
-__global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
+__global__ void __launch_bounds__(kBundleThreads, 1) k_bundle(const BundleArgs B) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long red_w[kBundleThreads / 32];
   __shared__ int red_k[kBundleThreads / 32];
   __shared__ double red_a[kBundleThreads / 32];
   __shared__ float red_s[kBundleThreads / 32];
   __shared__ Decision dec;
+  __shared__ int4 s_rec[3];  // DevNet::vdep of the fired reaction
 
   const RunArgs &r = B.r;
   const int M = r.net.M, N = r.net.N;
@@ -143,11 +164,14 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
   const int64_t k1 = min((int64_t)M, k0 + B.chunk);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int D = B.depth;
-  double *ring = (double *)smem;  // [D][3][kBundleThreads][2]: P, T, a pairs of each thread
-  int *Xs = (int *)(ring + (size_t)D * 3 * 2 * kBundleThreads);
+  // [D] stages of each thread's pairs: T, a (16 bytes each), the high words of P (8 bytes)
+  unsigned char *ring = smem;
+  int *Xs = (int *)(ring + (size_t)D * kStageBytes);
   uint32_t *bm = (uint32_t *)(Xs + N);
   const int nbm = (int)((B.chunk + 31) / 32);
-  double *P = B.P + j * B.Ms, *T = B.T + j * B.Ms, *A = B.A + j * B.Ms;
+  uint32_t *Ph = B.Ph + j * B.Ms, *Pl = B.Pl + j * B.Ms;
+  double *T = B.T + j * B.Ms, *A = B.A + j * B.Ms;
+  auto P_at = [&](int64_t k) { return __hiloint2double((int)Ph[k], (int)Pl[k]); };
   int32_t *NK = B.NK + j * B.Ms;
   Partial *part = B.part + j * 2 * C;
   unsigned long long *bar = B.bar + j;
@@ -173,7 +197,7 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
   int status = bad ? RT_TRAJ_BAD_X0 : RT_TRAJ_TEND;
   unsigned long long rounds = 0;
   float tau = __int_as_float(0x7F800000);
-  float tau_last = __int_as_float(0x7F800000);  // block thread 0: K / sum(a) at the last summed event
+  float tau_last = __int_as_float(0x7F800000);  // warp 0: K / sum(a) at the last summed event
   int64_t gi = 0;
   double next_g = 0.0;
   const int64_t tend_bits = dbits(r.t_end);
@@ -194,19 +218,25 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
     }
   };
 
-  // mark (set) or clear the slice bits of the channels that read a species changed by `mu`
-  auto touch_dependents = [&](int mu, bool set) {
-    const int vb = r.net.vptr[mu], ve = r.net.vptr[mu + 1];
-    for (int i = vb; i < ve; ++i) {
-      const int s = r.net.vlist[i].x;
-      const int qb = r.net.sptr[s], qe = r.net.sptr[s + 1];
-      for (int q = qb + tid; q < qe; q += blockDim.x) {
-        const int64_t rr = r.net.slist[q];
-        if (rr >= k0 && rr < k1) {
-          const int off = (int)(rr - k0);
-          if (set) atomicOr(&bm[off >> 5], 1u << (off & 31));
-          else bm[off >> 5] = 0u;
-        }
+  // mark the slice's channels that read a species the fired reaction changed; with a dependency
+  // record (in s_rec) the lists of all its species are read together
+  auto mark_dependents = [&](int mu) {
+    auto mark = [&](int32_t rr) {
+      if (rr >= k0 && rr < k1) {
+        const int off = (int)(rr - k0);
+        atomicOr(&bm[off >> 5], 1u << (off & 31));
+      }
+    };
+    if (r.net.vdep) {
+      const int4 vw = s_rec[0], rb = s_rec[1], rl = s_rec[2];
+      const int n0 = vpack_delta(vw.x) ? rl.x : 0, n1 = n0 + (vpack_delta(vw.y) ? rl.y : 0);
+      const int n2 = n1 + (vpack_delta(vw.z) ? rl.z : 0), n3 = n2 + (vpack_delta(vw.w) ? rl.w : 0);
+      for (int q = tid; q < n3; q += kBundleThreads)
+        mark(r.net.slist[q < n0 ? rb.x + q : q < n1 ? rb.y + (q - n0) : q < n2 ? rb.z + (q - n1) : rb.w + (q - n2)]);
+    } else {
+      for (int i = r.net.vptr[mu]; i < r.net.vptr[mu + 1]; ++i) {
+        const int s = r.net.vlist[i].x;
+        for (int q = r.net.sptr[s] + tid; q < r.net.sptr[s + 1]; q += kBundleThreads) mark(r.net.slist[q]);
       }
     }
   };
@@ -214,16 +244,22 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
   bool timed_out = false;
   if (!bad) {
     for (;;) {
-      // ---- fire the previous event's bookkeeping: new Exp(1) for P_mu (Eq. 27), dependents
-      if (mu_prev >= 0) {
-        if (tid == 0 && mu_prev >= k0 && mu_prev < k1) {
-          const int32_t n = NK[mu_prev] + 1;
-          NK[mu_prev] = n;
-          P[mu_prev] = __dadd_rn(P[mu_prev], exp1_draw(r.seed, g, (uint32_t)mu_prev, (uint32_t)n, r.stream_id));
-        }
-        touch_dependents(mu_prev, true);
-      }
+      // ---- the previous event's dependents are marked; the thread that scans the fired channel adds its
+      // new Exp(1) increment to P (Eq. 27) and uses the sum below, while the others begin the pass
+      int64_t k_new = -1;
+      uint32_t ph_new = 0;
+      if (mu_prev >= 0) mark_dependents(mu_prev);
       __syncthreads();
+      if (mu_prev >= k0 && mu_prev < k1 && ((mu_prev - k0) >> 1) % kBundleThreads == tid) {
+        const double Pk = P_at(mu_prev);
+        const int32_t n = NK[mu_prev] + 1;
+        NK[mu_prev] = n;
+        const double Pn = __dadd_rn(Pk, exp1_draw(r.seed, g, (uint32_t)mu_prev, (uint32_t)n, r.stream_id));
+        k_new = mu_prev;
+        ph_new = (uint32_t)__double2hiint(Pn);
+        Ph[mu_prev] = ph_new;
+        Pl[mu_prev] = (uint32_t)__double2loint(Pn);
+      }
 
       // ---- fused pass over the slice
       long long bestb = kInfBits;
@@ -243,14 +279,17 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
       const int64_t stride = 2 * (int64_t)blockDim.x;
       const int64_t kb = k0 + 2 * tid;
       const int nmine = kb < k1 ? (int)((k1 - kb + stride - 1) / stride) : 0;
-      auto slot = [&](int st, int arr) { return ring + ((size_t)(st * 3 + arr) * kBundleThreads + tid) * 2; };
+      // arr 0: T, 1: a (16 bytes), 2: the high words of P (8 bytes)
+      auto slot = [&](int st, int arr) {
+        return ring + (size_t)st * kStageBytes + (size_t)arr * 16 * kBundleThreads + (size_t)tid * (arr == 2 ? 8 : 16);
+      };
       int st_issue = 0, st_use = 0;
       auto issue = [&](int i) {  // pair i of this thread, one commit group (empty past the end)
         if (i < nmine) {
           const int64_t kk = kb + (int64_t)i * stride;
-          cp_async16(slot(st_issue, 0), P + kk);
-          cp_async16(slot(st_issue, 1), T + kk);
-          cp_async16(slot(st_issue, 2), A + kk);
+          cp_async16(slot(st_issue, 0), T + kk);
+          cp_async16(slot(st_issue, 1), A + kk);
+          cp_async8(slot(st_issue, 2), Ph + kk);
         }
         cp_async_commit();
         st_issue = st_issue + 1 == D ? 0 : st_issue + 1;
@@ -260,13 +299,13 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
         issue(i + D - 1);  // into the stage processed in the previous iteration
         cp_async_wait(D - 1);
         const int64_t k = kb + (int64_t)i * stride;
-        const double2 a2 = *(const double2 *)slot(st_use, 2);
-        const double2 t2 = *(const double2 *)slot(st_use, 1);
-        const double2 p2 = *(const double2 *)slot(st_use, 0);
+        const double2 a2 = *(const double2 *)slot(st_use, 1);
+        const double2 t2 = *(const double2 *)slot(st_use, 0);
+        const uint2 p2 = *(const uint2 *)slot(st_use, 2);
         st_use = st_use + 1 == D ? 0 : st_use + 1;
         const bool two = k + 1 < k1;
         double av[2] = {a2.x, a2.y}, tv[2] = {t2.x, t2.y};
-        const double pv[2] = {p2.x, p2.y};
+        const uint32_t pv[2] = {k == k_new ? ph_new : p2.x, k + 1 == k_new ? ph_new : p2.y};
         const uint32_t bits = bm[(k - k0) >> 5] >> ((k - k0) & 31);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -278,8 +317,10 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
           }
           if (dbits(av[h]) != 0) {
             if (summed) asum = __fadd_rn(asum, f32_lower(av[h]));
-            if (!exceeds(pv[h], tv[h], av[h], thr)) {
-              const long long wb = dbits(waiting_time(pv[h], tv[h], av[h]));
+            // the bounds read only the high words
+            if (!exceeds(__hiloint2double((int)pv[h], 0), tv[h], av[h], thr)) {
+              const double Pk = __hiloint2double((int)pv[h], (int)Pl[k + h]);
+              const long long wb = dbits(waiting_time(Pk, tv[h], av[h]));
               if (wb < bestb) {
                 bestb = wb;
                 bestk = (int)(k + h);
@@ -298,46 +339,36 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
 
       // ---- block argmin (lexicographic on (w, k)) and sum of a
       auto reduce_and_publish = [&](long long wb, int kk, double aa, float ss) {
+        const int src = warp_argmin(wb, kk);
+        if (summed)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const long long w2 = __shfl_xor_sync(0xFFFFFFFFu, wb, o);
-          const int k2 = __shfl_xor_sync(0xFFFFFFFFu, kk, o);
-          const double a2v = __shfl_xor_sync(0xFFFFFFFFu, aa, o);
-          ss = __fadd_rn(ss, __shfl_xor_sync(0xFFFFFFFFu, ss, o));
-          if (w2 < wb || (w2 == wb && (unsigned)k2 < (unsigned)kk)) {
-            wb = w2;
-            kk = k2;
-            aa = a2v;
-          }
-        }
-        if (lane == 0) {
+          for (int o = 16; o > 0; o >>= 1) ss = __fadd_rn(ss, __shfl_xor_sync(0xFFFFFFFFu, ss, o));
+        if (lane == src) {
           red_w[warp] = wb;
           red_k[warp] = kk;
           red_a[warp] = aa;
           red_s[warp] = ss;
         }
         __syncthreads();
-        if (tid == 0) {
-          long long w = red_w[0];
-          int k = red_k[0];
-          double a = red_a[0];
-          float s = red_s[0];
-          for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
-            if (red_w[i] < w || (red_w[i] == w && (unsigned)red_k[i] < (unsigned)k)) {
-              w = red_w[i];
-              k = red_k[i];
-              a = red_a[i];
-            }
-            s = __fadd_rn(s, red_s[i]);
+        if (warp == 0) {
+          const bool in = lane < kBundleThreads / 32;
+          const long long w = in ? red_w[lane] : kInfBits;
+          const int k = in ? red_k[lane] : -1;
+          float s = in ? red_s[lane] : 0.0f;
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) s = __fadd_rn(s, __shfl_xor_sync(0xFFFFFFFFu, s, o));
+          if (lane == warp_argmin(w, k)) {
+            Partial p;
+            p.wbits = w;
+            p.k = k;
+            p.pad = 0;
+            p.a = in ? red_a[lane] : 0.0;
+            p.asum = s;
+            p.pad2 = 0;
+            part[(rounds & 1) * C + c] = p;
+            if (r.net.vdep && k >= 0) prefetch_l2(r.net.vdep + 3 * (int64_t)k);
           }
-          Partial p;
-          p.wbits = w;
-          p.k = k;
-          p.pad = 0;
-          p.a = a;
-          p.asum = s;
-          p.pad2 = 0;
-          part[(rounds & 1) * C + c] = p;
+          __syncwarp();
         }
       };
       reduce_and_publish(bestb, bestk, besta, asum);
@@ -345,20 +376,20 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
       // ---- meet the other blocks of this trajectory; every block takes the same decision
       bool rescan_needed, rescanning = false;
       for (;;) {
-        if (tid == 0) {
+        if (warp == 0) {
           bool ok = true;
-          if (C > 1) ok = bundle_barrier(bar, (rounds + 1) * (unsigned long long)C, B.spin_limit);
-          dec.stop = 0;
-          dec.rescan = 0;
-          if (!ok) {
-            dec.stop = 1 + RT_TRAJ_TIMEOUT;
-          } else {
-            long long w = kInfBits;
-            int k = -1;
-            double a = 0.0;
-            float s = 0.0f;
-            const Partial *pp = part + (rounds & 1) * C;
-            for (int i = 0; i < C; ++i) {
+          if (C > 1) {
+            if (lane == 0) ok = bundle_barrier(bar, (rounds + 1) * (unsigned long long)C, B.spin_limit);
+            ok = __all_sync(0xFFFFFFFFu, ok);
+          }
+          // the C partials, a lane each; the same order of operations in every block
+          long long w = kInfBits;
+          int k = -1;
+          double a = 0.0;
+          float s = 0.0f;
+          const Partial *pp = part + (rounds & 1) * C;
+          if (ok)
+            for (int i = lane; i < C; i += 32) {
               const long long wi = __ldcg(&pp[i].wbits);
               const int ki = __ldcg(&pp[i].k);
               const double ai = __ldcg(&pp[i].a);
@@ -369,17 +400,23 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
                 a = ai;
               }
             }
-            if (summed && !rescanning) tau_last = s > 0.0f ? __fdiv_ru(kThresholdK, s) : __int_as_float(0x7F800000);
+          const int src = warp_argmin(w, k);
+          w = __shfl_sync(0xFFFFFFFFu, w, src);
+          k = __shfl_sync(0xFFFFFFFFu, k, src);
+          a = __shfl_sync(0xFFFFFFFFu, a, src);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) s = __fadd_rn(s, __shfl_xor_sync(0xFFFFFFFFu, s, o));
+          if (lane < 3 && r.net.vdep && k >= 0) s_rec[lane] = r.net.vdep[3 * (int64_t)k + lane];
+          if (summed && !rescanning) tau_last = s > 0.0f ? __fdiv_ru(kThresholdK, s) : __int_as_float(0x7F800000);
+          if (lane == 0) {
             // a threshold-filtered scan is exact only if its minimum is below the threshold
             const bool filtered = tau != __int_as_float(0x7F800000);
-            if (filtered && !(w < dbits((double)tau))) {
-              dec.rescan = 1;
-            } else {
-              dec.mu = k;
-              dec.dt = bitsd(w);
-              dec.a_mu = a;
-              dec.tau = tau_last;
-            }
+            dec.stop = ok ? 0 : 1 + RT_TRAJ_TIMEOUT;
+            dec.rescan = ok && filtered && !(w < dbits((double)tau)) ? 1 : 0;
+            dec.mu = k;
+            dec.dt = bitsd(w);
+            dec.a_mu = a;
+            dec.tau = tau_last;
           }
         }
         __syncthreads();
@@ -395,7 +432,7 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
         for (int64_t k = k0 + tid; k < k1; k += blockDim.x) {
           const double a = A[k];
           if (dbits(a) == 0) continue;
-          const double p = P[k], tt = T[k];
+          const double p = P_at(k), tt = T[k];
           if (bestb != kInfBits && exceeds(p, tt, a, f32_upper(bitsd(bestb)))) continue;
           const long long wb = dbits(waiting_time(p, tt, a));
           if (wb < bestb) {
@@ -412,8 +449,7 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
         status = RT_TRAJ_TIMEOUT;
         break;
       }
-      // clear this event's dependents bits before they change meaning
-      if (mu_prev >= 0) touch_dependents(mu_prev, false);
+      for (int w = tid; w < nbm; w += kBundleThreads) bm[w] = 0u;  // this event's marks are used up
 
       const int mu = dec.mu;
       if (mu < 0) {
@@ -430,17 +466,22 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
         status = RT_TRAJ_MAX_EVENTS;
         break;
       }
-      {
-        bool over = false;
+      bool over = false;
+      if (r.net.vdep) {
+        const int4 v = s_rec[0];
+        const int vw[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)  // a count past INT_MAX wraps below 0
+          if (vpack_delta(vw[i])) over |= (int)((uint32_t)Xs[vpack_species(vw[i])] + (uint32_t)vpack_delta(vw[i])) < 0;
+      } else {
         for (int i = r.net.vptr[mu]; i < r.net.vptr[mu + 1]; ++i) {
           const int2 e = r.net.vlist[i];
-          const long long nx = (long long)Xs[e.x] + e.y;
-          over |= (nx > INT_MAX) | (nx < 0);
+          over |= (int)((uint32_t)Xs[e.x] + (uint32_t)e.y) < 0;
         }
-        if (over) {
-          status = RT_TRAJ_OVERFLOW;
-          break;
-        }
+      }
+      if (over) {
+        status = RT_TRAJ_OVERFLOW;
+        break;
       }
       if (c == 0) {
         while (gi < r.G && dbits(next_g) < dbits(tn)) {
@@ -453,16 +494,22 @@ __global__ void __launch_bounds__(kBundleThreads) k_bundle(const BundleArgs B) {
       if (c == 0 && tid == 0) trace_event(r.out, j, ev, mu, tn);
       if (LL && c == 0 && tid == 0) ll = __dadd_rn(ll, rt_ln(dec.a_mu));
       __syncthreads();  // everyone has read Xs for this event
-      if (tid == 0)
+      if (r.net.vdep) {
+        if (tid < 4) {
+          const int w = ((const int *)s_rec)[tid];
+          if (vpack_delta(w)) Xs[vpack_species(w)] += vpack_delta(w);  // species are distinct within one reaction
+        }
+      } else if (tid == 0) {
         for (int i = r.net.vptr[mu]; i < r.net.vptr[mu + 1]; ++i) {
           const int2 e = r.net.vlist[i];
           Xs[e.x] += e.y;
         }
+      }
       ++ev;
       dprev = dmin;
       mu_prev = mu;
       tau = dec.tau;
-      __syncthreads();
+      // X, the cleared marks and the record are ordered by the barrier behind the next marking
     }
   }
   (void)timed_out;
@@ -537,7 +584,7 @@ static BundlePlan plan_bundle(const DevNet &net, int64_t n_traj, int C) {
   p.off_bar = off; off += (size_t)round_up(rows * sizeof(unsigned long long), 256);
   p.total = off;
   const size_t rest = (size_t)net.N * 4 + (size_t)((p.chunk + 31) / 32) * 4;
-  const size_t stage = (size_t)3 * 2 * kBundleThreads * 8;  // 24 KB per ring stage
+  const size_t stage = kStageBytes;  // 20 KB per ring stage
   int want = kRingDepth;  // RT_BUNDLE_RING_DEPTH (1..kMaxDepth) overrides, for tuning
   if (const char *env = getenv("RT_BUNDLE_RING_DEPTH")) want = std::min(kMaxDepth, std::max(1, atoi(env)));
   p.depth = 1;
@@ -606,7 +653,8 @@ int launch_bundle_mapping(const RunArgs &a, int ctas_per_traj, void *ws, size_t 
   B.C = C;
   B.Ms = p.Ms;
   B.chunk = p.chunk;
-  B.P = (double *)(w + p.off_P);
+  B.Ph = (uint32_t *)(w + p.off_P);
+  B.Pl = B.Ph + (a.n_traj > 0 ? a.n_traj : 1) * p.Ms;
   B.T = (double *)(w + p.off_T);
   B.A = (double *)(w + p.off_A);
   B.NK = (int32_t *)(w + p.off_NK);

@@ -143,11 +143,6 @@ __device__ __forceinline__ void st_cluster(uint32_t addr, unsigned long long v) 
   asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
 
-// a hint: bring the line holding p into L2 (no register result, never faults on a valid address)
-__device__ __forceinline__ void prefetch_l2(const void *p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
 __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ unsigned long long ld_mail(const unsigned long long *p) {
@@ -158,22 +153,6 @@ __device__ __forceinline__ unsigned long long ld_mail(const unsigned long long *
 
 __device__ __forceinline__ bool lex_less(long long w1, int k1, long long w2, int k2) {
   return w1 < w2 || (w1 == w2 && k1 < k2);
-}
-
-// lane of the lexicographic minimum of (w, k) over a warp, w >= 0 by its bits (every lane calls it)
-__device__ __forceinline__ int warp_argmin(long long w, int k) {
-  const uint32_t hi = (uint32_t)(w >> 32), mh = __reduce_min_sync(0xFFFFFFFFu, hi);
-  unsigned b = __ballot_sync(0xFFFFFFFFu, hi == mh);
-  if (b & (b - 1)) {
-    const uint32_t lo = hi == mh ? (uint32_t)w : 0xFFFFFFFFu, ml = __reduce_min_sync(0xFFFFFFFFu, lo);
-    b = __ballot_sync(0xFFFFFFFFu, hi == mh && lo == ml);
-    if (b & (b - 1)) {
-      const bool in = hi == mh && lo == ml;
-      const uint32_t mk = __reduce_min_sync(0xFFFFFFFFu, in ? (uint32_t)k : 0xFFFFFFFFu);
-      b = __ballot_sync(0xFFFFFFFFu, in && (uint32_t)k == mk);
-    }
-  }
-  return __ffs((int)b) - 1;
 }
 
 // a warp's candidate for the slice minimum; its dependency record is copied here asynchronously when

@@ -252,4 +252,26 @@ __device__ __forceinline__ T pick(const T (&v)[R], int r) {
   return out;
 }
 
+// lane of the lexicographic minimum of (w, k) over a warp, w >= 0 by its bits, k as an
+// unsigned number (every lane calls it)
+__device__ __forceinline__ int warp_argmin(long long w, int k) {
+  const uint32_t hi = (uint32_t)(w >> 32), mh = __reduce_min_sync(0xFFFFFFFFu, hi);
+  unsigned b = __ballot_sync(0xFFFFFFFFu, hi == mh);
+  if (b & (b - 1)) {
+    const uint32_t lo = hi == mh ? (uint32_t)w : 0xFFFFFFFFu, ml = __reduce_min_sync(0xFFFFFFFFu, lo);
+    b = __ballot_sync(0xFFFFFFFFu, hi == mh && lo == ml);
+    if (b & (b - 1)) {
+      const bool in = hi == mh && lo == ml;
+      const uint32_t mk = __reduce_min_sync(0xFFFFFFFFu, in ? (uint32_t)k : 0xFFFFFFFFu);
+      b = __ballot_sync(0xFFFFFFFFu, in && (uint32_t)k == mk);
+    }
+  }
+  return __ffs((int)b) - 1;
+}
+
+// a hint: bring the line holding p into L2 (no register result, never faults on a valid address)
+__device__ __forceinline__ void prefetch_l2(const void *p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
 }  // namespace rt
