@@ -4,6 +4,7 @@
 // block.  Beside it Table 3's form with a lane per channel.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -22,8 +23,8 @@ static size_t warp_moment_bytes(const RunArgs &a) {
 
 // Start of the trajectories' state in a block's shared memory, after the network's tables and the
 // moment table.
-__host__ __device__ inline size_t warp_state_off(int M, int nv, int64_t nmom, bool td) {
-  const size_t b = (size_t)M * (8 + 8 + (td ? 8 : 0)) + (size_t)nv * 8 + (size_t)nmom * 8 + (size_t)(M + 1) * 4;
+__host__ __device__ inline size_t warp_state_off(int M, int nv, int64_t nmom, bool td, bool copy) {
+  const size_t b = (size_t)M * (8 + 8 + (td ? 8 : 0)) + (size_t)nv * 8 + (size_t)nmom * 8 + (copy ? (size_t)(M + 1) * 4 : 0);
   return (b + 127) / 128 * 128;
 }
 
@@ -31,14 +32,17 @@ __host__ __device__ inline size_t warp_state_off(int M, int nv, int64_t nmom, bo
 // 65536 trajectories of 64 reactions with likelihood and gradient 350 -> 186 ms, 10000 trajectories of 200
 // reactions with moments 74.8 -> 51.8 ms; time-dependent rates against every root exactly with one
 // trajectory per warp: 10000 trajectories of 48 reactions 83 -> 26 ms.
-template <int R, int G, bool LL, bool TD>
+// COPY: the net changes in shared memory too (else, read once per event, in global memory: where their
+// copies would keep a block off the SM -- 200 reactions, 5 instead of 6 blocks, 47.6 -> 45.5 ms; with
+// the blocks that fit unchanged the copies are the better place, 64 reactions 180 against 207 ms).
+template <int R, int G, bool LL, bool TD, bool COPY>
 __global__ void __launch_bounds__(kWarpBlock, 6)
     k_ens_warp(const RunArgs A, const int tend_finite, const int use_mom) {
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int S = 32 / G;  // trajectories per warp
   const DevNet &d = A.net;
-  const int M = d.M, N = d.N, nv = TD ? 0 : d.n_vnz;
-  // carve: c[M], beta[M] (TD), rd[M], vl[nv], moments, vp[M+1], the trajectories
+  const int M = d.M, N = d.N, nv = COPY ? d.n_vnz : 0;
+  // carve: c[M], beta[M] (TD), rd[M], vl[nv] (COPY), moments, vp[M+1] (COPY), the trajectories
   double *s_c = (double *)smem;
   double *s_beta = s_c + M;
   int2 *s_rd = (int2 *)(s_beta + (TD ? M : 0));
@@ -47,17 +51,18 @@ __global__ void __launch_bounds__(kWarpBlock, 6)
   const int64_t GN = A.G * N;
   const int64_t nmom = use_mom ? 2 * GN + A.G : 0;
   int *s_vp = (int *)(s_mom + nmom);
-  unsigned char *s_state = smem + warp_state_off(M, nv, nmom, TD);
+  unsigned char *s_state = smem + warp_state_off(M, nv, nmom, TD, COPY);
   for (int i = threadIdx.x; i < M; i += blockDim.x) {
     s_c[i] = d.c[i];
     s_rd[i] = d.rdesc[i];
     if (TD) s_beta[i] = d.beta[i];
   }
   for (int i = threadIdx.x; i < nv; i += blockDim.x) s_vl[i] = d.vlist[i];
-  for (int i = threadIdx.x; i <= M; i += blockDim.x) s_vp[i] = d.vptr[i];
+  if (COPY)
+    for (int i = threadIdx.x; i <= M; i += blockDim.x) s_vp[i] = d.vptr[i];
   for (int64_t i = threadIdx.x; i < nmom; i += blockDim.x) s_mom[i] = 0ull;
   __syncthreads();
-  const WarpNet net{M, N, s_rd, s_c, s_vp, TD ? d.vlist : s_vl, d.dptr, d.dlist, s_beta};
+  const WarpNet net{M, N, s_rd, s_c, COPY ? s_vp : d.vptr, COPY ? s_vl : d.vlist, d.dptr, d.dlist, s_beta};
   const int warp = threadIdx.x >> 5;
   const int64_t j0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * S;
   if (j0 < A.n_traj)
@@ -340,24 +345,45 @@ int launch_rescaled_warp_mapping(const RunArgs &a, int lanes_per_traj, cudaStrea
 
 int warp_mapping_max_m() { return 256; }
 
-template <int R, int G, bool TD>
-static cudaError_t launch_rg(const RunArgs &a, cudaStream_t s, int tend_finite) {
+template <int R, int G, bool TD, bool COPY>
+static cudaError_t launch_rgc(const RunArgs &a, cudaStream_t s, int tend_finite) {
   constexpr int S = 32 / G;
   const size_t per_warp = S * warp_seg_bytes(a.net.M, a.net.N, G);
-  const int nv = TD ? 0 : a.net.n_vnz;  // TD reads the net changes from global memory
+  const int nv = COPY ? a.net.n_vnz : 0;
   size_t mom = warp_moment_bytes(a);
-  if (warp_state_off(a.net.M, nv, (int64_t)(mom / 8), TD) + per_warp > kWarpSmemMax) mom = 0;  // added in global memory
-  const size_t off = warp_state_off(a.net.M, nv, (int64_t)(mom / 8), TD);
+  if (warp_state_off(a.net.M, nv, (int64_t)(mom / 8), TD, COPY) + per_warp > kWarpSmemMax) mom = 0;  // added in global memory
+  const size_t off = warp_state_off(a.net.M, nv, (int64_t)(mom / 8), TD, COPY);
   int wpb = kWarpBlock / 32;  // fewer warps per block where many species or moments leave no room
   while (wpb > 1 && off + wpb * per_warp > kWarpSmemMax) wpb /= 2;
   const size_t smem = off + wpb * per_warp;
   const int64_t per_block = (int64_t)wpb * S;
   if ((a.n_traj + per_block - 1) / per_block > INT_MAX) return cudaErrorInvalidConfiguration;
   const unsigned grid = (unsigned)((a.n_traj + per_block - 1) / per_block);
-  auto kern = a.out.loglik_dev ? k_ens_warp<R, G, true, TD> : k_ens_warp<R, G, false, TD>;
+  auto kern = a.out.loglik_dev ? k_ens_warp<R, G, true, TD, COPY> : k_ens_warp<R, G, false, TD, COPY>;
   raise_smem_limit((const void *)kern, smem);
   kern<<<grid, wpb * 32, smem, s>>>(a, tend_finite, mom ? 1 : 0);
   return cudaGetLastError();
+}
+
+// Blocks of four warps that an SM's shared memory holds (1 KB of each is the system's), at most the six
+// that the registers allow.
+template <int G, bool TD>
+static int blocks_that_fit(const RunArgs &a, bool copy) {
+  const size_t mom = warp_moment_bytes(a);
+  const size_t b = warp_state_off(a.net.M, copy ? a.net.n_vnz : 0, (int64_t)(mom / 8), TD, copy) +
+                   kWarpBlock / 32 * (32 / G) * warp_seg_bytes(a.net.M, a.net.N, G);
+  return (int)std::min<size_t>(6, (228 * 1024) / (b + 1024));
+}
+
+template <int R, int G, bool TD>
+static cudaError_t launch_rg(const RunArgs &a, cudaStream_t s, int tf) {
+  // only the widest networks' copies can cost a block; TD's net changes may not fit at all
+  if constexpr (TD || (R == 8 && G == 32)) {
+    if (TD || blocks_that_fit<G, TD>(a, true) < blocks_that_fit<G, TD>(a, false))
+      return launch_rgc<R, G, TD, false>(a, s, tf);
+  }
+  if constexpr (TD) return cudaErrorInvalidConfiguration;  // not reached
+  else return launch_rgc<R, G, false, true>(a, s, tf);
 }
 
 template <bool TD>
@@ -425,7 +451,7 @@ int launch_tdep_warp_mapping(const RunArgs &a, int lanes_per_traj, cudaStream_t 
   if ((a.n_traj + kWarpBlock / 32 - 1) / (kWarpBlock / 32) > INT_MAX)
     return set_error(RT_ERR_UNSUPPORTED, "warp mapping: too many trajectories for one launch");
   int G = choose_lanes(M, lanes_per_traj);
-  if (warp_state_off(M, 0, 0, true) + (32 / G) * warp_seg_bytes(M, a.net.N, G) > kWarpSmemMax) G = 32;  // many species
+  if (warp_state_off(M, 0, 0, true, false) + (32 / G) * warp_seg_bytes(M, a.net.N, G) > kWarpSmemMax) G = 32;  // many species
   const cudaError_t e = launch_g<true>(a, G, s, std::isfinite(a.t_end) ? 1 : 0);
   if (e != cudaSuccess) return set_error(RT_ERR_CUDA, "time-dependent warp kernel launch: %s", cudaGetErrorString(e));
   return RT_OK;
