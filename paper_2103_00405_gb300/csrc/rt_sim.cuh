@@ -217,13 +217,6 @@ __device__ __forceinline__ float wait_interval(float2 b, double T, float &lo) {
 // of the exact operations are below 2^-17.
 __device__ __forceinline__ float interval_threshold(float ub) { return __fmul_ru(fmaxf(ub, 0.0f), 1.00000763f); }
 
-// An estimate of (P - T) / a used only to choose the candidate that is computed
-// exactly first (any choice gives the same, exact result).
-__device__ __forceinline__ float wait_estimate(double P, double T, double a) {
-  const float rem = f32_upper(P) - f32_lower(T);
-  return rem > 0.0f ? __fdividef(rem, f32_lower(a) + 1e-37f) : 0.0f;
-}
-
 // Per-event trace: event ev of trajectory j fired channel mu at time t (recorded for
 // the first trace_len events).
 __device__ __forceinline__ void trace_event(const rt_outputs &o, int64_t j, int32_t ev, int mu, double t) {
