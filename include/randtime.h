@@ -60,10 +60,11 @@ enum {
 /* Trajectory-to-hardware mappings. */
 enum {
   RT_MAP_AUTO = -1,  /* chosen by the library from the network size */
-  RT_MAP_THREAD = 0, /* one thread per trajectory, state in registers (M <= 16; with M <= 4 and
-                        N <= 4 the counts and the network too) */
+  RT_MAP_THREAD = 0, /* one thread per trajectory (M <= 16; with M <= 4 and N <= 4 the counts and
+                        the network in registers too).  Left to the library (RT_MAP_AUTO), few
+                        trajectories of such networks run a warp each, a lane per channel */
   RT_MAP_WARP = 1,   /* a warp segment (8, 16 or 32 lanes) per trajectory, channels spread over lanes */
-  RT_MAP_BLOCK = 2,  /* one thread block per trajectory, state in registers (M <= 8 * block_threads) */
+  RT_MAP_BLOCK = 2,  /* one thread block per trajectory, state on chip (M <= 8 * block_threads) */
   RT_MAP_BUNDLE = 3, /* several blocks per trajectory, state streamed through HBM */
   RT_MAP_TREE = 4    /* absolute-time form only: a thread-block cluster per trajectory, min-tree
                         argmin, only the channels an event touches updated */
@@ -191,8 +192,8 @@ int rt_network_set_enabled(rt_network *net, const uint8_t *enabled);
  * u = 1 + beta_k t, b = A_k u, R = P_k - T_k (for beta_k = 0: R / A_k, the constant-rate
  * operations); ln a_mu is taken at the event time.  The gradient (n_k - T_k) / c_k keeps
  * its form.  Networks with slopes run the internal-time form on the thread mapping
- * (M <= 16) or the warp mapping (M <= 256, 32 lanes per trajectory; the default above
- * 16 reactions); other mappings, forms and batches return RT_ERR_UNSUPPORTED.  Copies to
+ * (M <= 16) or the warp mapping (M <= 256; the default above 16 reactions;
+ * lanes_per_traj 0 or 32); other mappings, forms and batches return RT_ERR_UNSUPPORTED.  Copies to
  * the device synchronously; no work using the network may be in flight.
  */
 int rt_network_set_rate_slopes(rt_network *net, const double *beta);

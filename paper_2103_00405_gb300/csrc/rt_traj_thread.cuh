@@ -1,9 +1,10 @@
-// rt_traj_thread.cuh -- one thread per trajectory, state in registers.
+// rt_traj_thread.cuh -- one thread per trajectory.
 //
 // The NRRTA loop of Table 2 (Liu & Wang, arXiv:2103.00405) in internal-time form:
-// a thread keeps its trajectory's P_k, T_k and a_k (Eq. 17-25) for all M <= 16
-// channels in registers and its counts X in shared memory (a column per thread,
-// X[s] at X[s * B], so accesses are bank-conflict free).  The network tables
+// a thread keeps its trajectory's P_k, T_k and a_k (Eq. 17-25) in registers
+// (simulate_one) or, for 5 to 16 channels, in shared memory (simulate_mid), and its
+// counts X in shared memory (a column per thread, X[s] at X[s * B], so accesses are
+// bank-conflict free).  The network tables
 // (reactant descriptors, rates, net changes, per-reaction dependency masks) are
 // reached through generic pointers: shared memory in the single-network kernel,
 // global memory in the batched kernel.
