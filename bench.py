@@ -10,7 +10,7 @@ their own disjoint blocks), and the int64 moment sums are all-reduced over ranks
 
 `workloads` (same JSON line, each with its own small fixed step count):
   large   -- random network N = 1e4, M = 1e6, 16 trajectories, a bundle of blocks per
-             trajectory streaming P, T, a through HBM (HBM roofline, 32 B per
+             trajectory streaming P, T, a through HBM (HBM roofline, 28 B per
              channel-event); --events events per trajectory per step
   large_tree -- the same network as configured (16 trajectories x 1e6 events) in the
              absolute-time form: a thread-block cluster per trajectory, min-tree argmin
@@ -235,25 +235,13 @@ class ClockSampler:
 # Roofline arithmetic
 # ----------------------------------------------------------------------------------------
 
-def dependents_per_channel(net) -> np.ndarray:
-    """For every channel k, how many propensities its firing recomputes: the channels reading a
-    species k changes, counted once per (changed species, reading channel) pair."""
-    readers = np.zeros(net.n_species, np.int64)
-    np.add.at(readers, net.reac_sp, 1)
-    deps = np.zeros(net.n_reactions, np.int64)
-    np.add.at(deps, net.stoi_rxn, readers[net.stoi_sp])
-    return deps
-
-
-def fp64_ops_per_event(net, counts):
-    """Algorithmic binary64 operations of the events (Table 2 with Eq. 17, 25): per event and
-    channel P-T, /a, a*dt, T+ (4); per event t+dt and P_mu+E (2); a conversion and a multiply
-    for every propensity the fired channel recomputes.  counts: [M] firings over the launch.
-    Returns (operations, events)."""
-    deps = dependents_per_channel(net)
-    M = net.n_reactions
+def fp64_ops_per_event(net, counts, per_channel):
+    """Binary64 operations of the events that run on the FP64 pipe (Table 2 with Eq. 17, 25): per event
+    and channel a*dt and T+ (2), in the one-thread kernels P-T as well (3; the others bound it in floats);
+    per event t+dt and P_mu+E (2).  Quotients, propensities and logarithms are integer work.  counts: [M]
+    firings over the launch.  Returns (operations, events)."""
     n = float(np.sum(counts))
-    return float(n * (4 * M + 2) + 2 * float(np.dot(counts, deps))), n
+    return float(n * (per_channel * net.n_reactions + 2)), n
 
 
 def hbm_peak_gbs():
@@ -467,11 +455,10 @@ def run_ensemble(args, ctx):
                        traj_offset=traj_base(ctx.rank, args.steps - 1, n), grad=True, mapping=L.RT_MAP_THREAD,
                        max_events=cfgs[0]["max_events"])
     counts = chk["counts"].sum(0, dtype=torch.int64).cpu().numpy()
-    ops_s, ev_s = fp64_ops_per_event(cfgs[0]["net"], counts)
+    ops_s, ev_s = fp64_ops_per_event(cfgs[0]["net"], counts, 3)
     lv_events = int(outs[0]["n_events"].sum().item())
     roof = alu_roofline(ops_s / ev_s * lv_events, lv_ms[-1], ctx.fp64_peak, "k_ens_small<3,2,false> "
-                        "(Lotka-Volterra launch)", "%.3f algorithmic FP64 ops per event (4M+2 + 2 per recomputed "
-                        "propensity)" % (ops_s / ev_s))
+                        "(Lotka-Volterra launch)", "%.3f FP64 ops per event (3M+2)" % (ops_s / ev_s))
     tr = NCU_TRAFFIC["k_ens_small"]
     roof["traffic"] = tr["bytes_per_unit"] * n if tr["bytes_per_unit"] else None
     roof["traffic_note"] = tr["source"] + ", scaled to this launch's trajectories"
@@ -562,7 +549,7 @@ def run_large(args, ctx, steps, warmup):
     dev_ms, events_all = combine_over_ranks(sum(ms), events, ctx.world, ctx.dev)
     peak, how = hbm_peak_gbs()
     per_launch_events = events / steps
-    achieved = 32.0 * M * per_launch_events / (statistics.mean(ms) / 1e3) / 1e9
+    achieved = 28.0 * M * per_launch_events / (statistics.mean(ms) / 1e3) / 1e9
     tr = NCU_TRAFFIC["k_bundle"]
     return {"value": events_all / (dev_ms / 1e3), "unit": UNIT, "steps": steps, "warmup": warmup,
             "ms_per_step": dev_ms / steps,
@@ -579,7 +566,7 @@ def run_large(args, ctx, steps, warmup):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": (tr["bytes_per_unit"] * M * per_launch_events if tr["bytes_per_unit"] else None),
                          "traffic_note": tr["source"] + ", scaled to this launch's channel-events",
-                         "kernel": "k_bundle<false>", "bytes_per_channel_event": 32, "peak_source": how}}
+                         "kernel": "k_bundle<false>", "bytes_per_channel_event": 28, "peak_source": how}}
 
 
 def distinct_dependents(net, channels) -> np.ndarray:
@@ -758,13 +745,12 @@ def run_batched(args, ctx, steps, warmup):
     events = int(ev_net.sum())
     dev_ms, events_all = combine_over_ranks(sum(ms), events * steps, ctx.world, ctx.dev)
 
-    # algorithmic FP64 operations: per event of network i, 4 M_i + 2, plus 2 per recomputed
-    # propensity with the mean dependents count of the network's channels
+    # FP64 operations: per event of network i, 2 M_i + 2
     ops = 0.0
     for it, e in zip(items, ev_net):
-        ops += float(e) * (4 * it.net.n_reactions + 2 + 2 * float(dependents_per_channel(it.net).mean()))
+        ops += float(e) * (2 * it.net.n_reactions + 2)
     roof = alu_roofline(ops, statistics.mean(ms), ctx.fp64_peak, "k_batch<false> (persistent, graph-captured)",
-                        "per event of network i: 4 M_i + 2 + 2 x mean dependents of its channels")
+                        "per event of network i: 2 M_i + 2 (T += a dt of every channel)")
 
     line = {"value": events_all / (dev_ms / 1e3), "unit": UNIT, "steps": steps, "warmup": warmup,
             "ms_per_step": dev_ms / steps,
@@ -864,11 +850,11 @@ def run_grad(args, ctx, steps, warmup):
     dev_ms, events_all = combine_over_ranks(sum(ms), events * steps, ctx.world, ctx.dev)
     pms, _ = combine_over_ranks(sum(ms_plain), 0, ctx.world, ctx.dev)
     counts = out_grad["counts"].sum(0, dtype=torch.int64).cpu().numpy()
-    ops, ev = fp64_ops_per_event(net, counts)
+    ops, ev = fp64_ops_per_event(net, counts, 2)
     fwd_ms = statistics.mean(m["forward"] for m in marks)
     roof = alu_roofline(ops, fwd_ms, ctx.fp64_peak, "k_ens_warp<8,8,true> (8 lanes per trajectory, forward with the log-likelihood)",
-                        "%.1f algorithmic FP64 ops per event (4M+2 + 2 per recomputed propensity; the "
-                        "fixed-point logarithms are integer work)" % (ops / ev))
+                        "%.1f FP64 ops per event (2M+2; quotients, propensities and logarithms are integer "
+                        "work)" % (ops / ev))
     return {"value": events_all / (dev_ms / 1e3), "unit": UNIT, "steps": steps, "warmup": warmup,
             "ms_per_step": dev_ms / steps,
             "config": {"workload": "gradient: random network M=64, N=16, c~lognormal(0,0.5), X0~Poisson(200), "
