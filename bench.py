@@ -61,12 +61,12 @@ FP64_OP_NOMINAL = 0.625e12
 # (dram__bytes_read.sum + dram__bytes_write.sum of one launch over the units it
 # processed).  A kernel changed since its capture must have its entry set to None.
 NCU_TRAFFIC = {
-    "k_bundle": dict(bytes_per_unit=(77562891264 + 25620826880) / (200 * 16 * 1e6), unit="channel-event",
-                     source="ncu capture of k_bundle<false>, N=1e4, M=1e6, 16 trajectories x 200 events"),
+    "k_bundle": dict(bytes_per_unit=(19653502208 + 7660353792) / (60 * 16 * 1e6), unit="channel-event",
+                     source="ncu capture of k_bundle<false>, N=1e4, M=1e6, 16 trajectories x 60 events"),
     "k_ens_small": dict(bytes_per_unit=(818944 + 0) / 16384, unit="trajectory",
                         source="ncu capture of k_ens_small<3,2,false>, 16384 Lotka-Volterra trajectories to t=10"),
-    "k_lazy": dict(bytes_per_unit=(2468666880 + 874632704) / (16 * 2000), unit="event",
-                   source="ncu capture of k_lazy<false>, N=1e4, M=1e6, 16 trajectories x 2000 events"),
+    "k_lazy": dict(bytes_per_unit=(3024477696 + 649416448) / (16 * 1500), unit="event",
+                   source="ncu capture of k_lazy<false, true>, N=1e4, M=1e6, 16 trajectories x 1500 events"),
 }
 
 
@@ -561,7 +561,7 @@ def run_large(args, ctx, steps, warmup):
                                "run for %d events each; the 1e6-event runs of the configuration take 10 such "
                                "steps" % args.events,
                        "t_end": "inf", "seed": 1, "parallelism": "replicas" if ctx.world > 1 else "1 GPU",
-                       "l2": "inputs larger than L2 (16 x 24 MB of P, T, a streamed per event)"},
+                       "l2": "inputs larger than L2 (16 x 20 MB of P, T, a streamed per event)"},
             "events_per_step": events_all / steps, "clocks": clocks, "gpu_launches": 2 * steps,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": (tr["bytes_per_unit"] * M * per_launch_events if tr["bytes_per_unit"] else None),
