@@ -381,6 +381,7 @@ __global__ void __launch_bounds__(kBundleThreads, 1) k_bundle(const BundleArgs B
           if (C > 1) {
             if (lane == 0) ok = bundle_barrier(bar, (rounds + 1) * (unsigned long long)C, B.spin_limit);
             ok = __all_sync(0xFFFFFFFFu, ok);
+            __syncwarp();  // lane 0 acquired; the other lanes' loads of the partials come after (a vote orders no memory)
           }
           // the C partials, a lane each; the same order of operations in every block
           long long w = kInfBits;

@@ -61,3 +61,11 @@ def test_overflow_is_not_fired():
     x0[s] = 2**31 - 5
     o = check(base.with_rates(c), x0, max_events=50, ctas_per_traj=2)
     assert (o["status"] == oracle.ST_OVERFLOW).any() or (o["n_events"] > 0).any()
+
+
+@pytest.mark.parametrize("ctas", [2, 32, 33, 65, 152])
+def test_every_lane_reads_the_partials_of_its_event(ctas):
+    """One, several or no partial minima per lane, exchanged a few thousand times: a lane that read a partial
+    of an earlier event would leave the oracle's path."""
+    net = W.random_mass_action(600, 152 * 32, 77, 1.0)
+    check(net, W.poisson_x0(600, 40, 5), n_traj=1 if ctas > 76 else 2, max_events=2000, ctas_per_traj=ctas)
