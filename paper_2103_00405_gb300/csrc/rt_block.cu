@@ -38,6 +38,9 @@ static cudaError_t launch_r(const RunArgs &a, int B, cudaStream_t s, int tf) {
   return cudaGetLastError();
 }
 
+// The fewest threads of a block left to the library: one for eight channels.
+static int fewest_threads(int M) { return std::min(512, std::max(64, ((M + 7) / 8 + 31) / 32 * 32)); }
+
 // Threads per trajectory: between one for eight channels and one each, as many as let the SM's share of
 // the trajectories be resident at 64 registers (1024 threads).  A block with few slots per thread takes
 // fewer instructions one after the other per event; with many, more trajectories share the SM.
@@ -46,9 +49,9 @@ static int choose_threads(int M, int64_t n_traj) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t per_sm = std::max<int64_t>(1, (n_traj + sms - 1) / std::max(1, sms));
-  const int lo = std::max(64, ((M + 7) / 8 + 31) / 32 * 32), hi = std::min(512, (M + 31) / 32 * 32);
+  const int hi = std::min(512, (M + 31) / 32 * 32);
   const int fit = (int)std::max<int64_t>(0, 1024 / per_sm) / 32 * 32;
-  return std::min(512, std::max(lo, std::min(hi, fit)));
+  return std::max(fewest_threads(M), std::min(hi, fit));
 }
 
 int launch_block_mapping(const RunArgs &a, int block_threads, cudaStream_t s) {
@@ -59,8 +62,11 @@ int launch_block_mapping(const RunArgs &a, int block_threads, cudaStream_t s) {
   if (B % 32 || B > 512) return set_error(RT_ERR_INVALID_ARG, "block mapping: block_threads must be a multiple of 32 <= 512");
   const int R = (M + B - 1) / B;
   if (R > 8) return set_error(RT_ERR_UNSUPPORTED, "block mapping supports M <= 8 * block_threads (M = %d)", M);
-  // at most 200 KB for X, counts and the reductions' 24 bytes a warp and 8 a thread
-  if ((size_t)a.net.N * 4 + (size_t)M * 4 + (size_t)((M + 31) / 32) * 4 + (size_t)(B / 32) * 24 + (size_t)B * 8 + 96 >
+  // What is refused: more than 200 KB for X, the counts, the bitmap and an allowance of 24 bytes a warp and 8
+  // a thread.  A block size left to the library is taken as the smallest, so that the number of trajectories
+  // does not decide; the scratch that is launched (40 bytes a thread) is at most 20 KB more and fits.
+  const int Bf = block_threads > 0 ? B : fewest_threads(M);
+  if ((size_t)a.net.N * 4 + (size_t)M * 4 + (size_t)((M + 31) / 32) * 4 + (size_t)(Bf / 32) * 24 + (size_t)Bf * 8 + 96 >
       200 * 1024)
     return set_error(RT_ERR_UNSUPPORTED, "block mapping: %d species do not fit in shared memory", a.net.N);
   const int tf = std::isfinite(a.t_end) ? 1 : 0;

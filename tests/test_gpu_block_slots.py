@@ -60,3 +60,21 @@ def test_batch_of_every_class(block_threads, n_big):
                  t_last=out["t_last"][i], loglik=out["loglik"][i], counts=batch.per_channel_of(out, "counts", i, nt),
                  t_internal=batch.per_channel_of(out, "t_internal", i, nt))
         assert_same(g, o)
+
+
+@pytest.mark.parametrize("n_traj", [1, 153, 1300])
+def test_species_limit_does_not_depend_on_the_trajectories(n_traj):
+    """The most species that the smallest block (64 threads here) is given run with every number of
+    trajectories, one more is refused with every number."""
+    m, b = 300, 64
+    n = (200 * 1024 - m * 4 - (m + 31) // 32 * 4 - b // 32 * 24 - b * 8 - 96) // 4
+    net = W.random_mass_action(n, m, 71, 0.7)
+    x0 = np.random.default_rng(2).poisson(20, n).astype(np.int32)
+    kw = dict(seed=4, max_events=40)
+    g = api.simulate(api.Network(net), x0, 1.0, n_traj, grad=True, **kw)
+    few = min(n_traj, 3)
+    o = oracle.run(net, x0, 1.0, few, want_grad=True, n_threads=4, **kw)
+    assert_same({k: v[:few] for k, v in g.items() if not k.startswith("_")}, o)
+    wide = W.random_mass_action(n + 1, m, 71, 0.7)
+    with pytest.raises(L.RandtimeError):
+        api.simulate(api.Network(wide), np.zeros(n + 1, np.int32), 1.0, n_traj, **kw)
