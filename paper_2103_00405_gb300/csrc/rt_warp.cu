@@ -439,6 +439,20 @@ int launch_warp_mapping(const RunArgs &a, int block_threads, int lanes_per_traj,
   return RT_OK;
 }
 
+// Where time-dependent rates take 32 lanes per trajectory whatever the network's size.
+// Few trajectories (12 an SM): every trajectory's warp is resident, an event's latency counts, and each further
+// channel per lane is a part of it.  300 events, 32 lanes / the width by M: 32 reactions 100 trajectories 0.88 /
+// 1.63 ms, 1824 1.27 / 1.64, 2432 1.65 / 1.63; 64 reactions 1.01 / 2.28, 1.52 / 2.29, 2.00 / 2.29; 128 reactions
+// 1.27 / 2.06, 2.14 / 2.66, 2.85 / 2.67.
+// So many species that a block of narrower segments, each with its own X, holds fewer than four warps: 10000
+// trajectories, 9000 species: 20 reactions 7.1 / 11.7 ms, 64 reactions 8.4 / 17.6, 128 reactions 10.9 / 16.7.
+constexpr int64_t kTdepWideTraj = 152 * 12;
+static bool tdep_wide(const RunArgs &a, int G) {
+  const size_t block = warp_state_off(a.net.M, 0, 0, true, false) +
+                       kWarpBlock / 32 * (32 / G) * warp_seg_bytes(a.net.M, a.net.N, G);
+  return a.n_traj <= kTdepWideTraj || block > kWarpSmemMax;
+}
+
 int launch_tdep_warp_mapping(const RunArgs &a, int lanes_per_traj, cudaStream_t s) {
   if (a.n_traj == 0) return RT_OK;
   const int M = a.net.M;
@@ -451,7 +465,7 @@ int launch_tdep_warp_mapping(const RunArgs &a, int lanes_per_traj, cudaStream_t 
   if ((a.n_traj + kWarpBlock / 32 - 1) / (kWarpBlock / 32) > INT_MAX)
     return set_error(RT_ERR_UNSUPPORTED, "warp mapping: too many trajectories for one launch");
   int G = choose_lanes(M, lanes_per_traj);
-  if (warp_state_off(M, 0, 0, true, false) + (32 / G) * warp_seg_bytes(M, a.net.N, G) > kWarpSmemMax) G = 32;  // many species
+  if (tdep_wide(a, G)) G = 32;
   const cudaError_t e = launch_g<true>(a, G, s, std::isfinite(a.t_end) ? 1 : 0);
   if (e != cudaSuccess) return set_error(RT_ERR_CUDA, "time-dependent warp kernel launch: %s", cudaGetErrorString(e));
   return RT_OK;

@@ -1,0 +1,44 @@
+"""What the library chooses by itself is not slower than what a caller can name: the same call timed both ways on
+the device, the shorter of several runs of each.  The lines of these choices were measured; a tenth is allowed."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2103_00405_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - CPU-only hosts skip the GPU suite
+    pytest.skip("CUDA not available", allow_module_level=True)
+
+from paper_2103_00405_gb300 import api  # noqa: E402
+
+
+def ms(fn, runs=7):
+    fn()
+    best = float("inf")
+    for _ in range(runs):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        fn()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("n_traj", [20, 600, 1800])
+@pytest.mark.parametrize("m", [17, 32, 64, 100])
+def test_ramped_segment_width_by_trajectories(m, n_traj):
+    n = max(4, m // 4)
+    net = api.Network(W.random_mass_action(n, m, W.GEN_SEED_BASE + m, 0.5))
+    rng = np.random.default_rng(m)
+    net.set_rate_slopes(np.where(rng.random(m) < 0.3, 0.0, rng.uniform(0.1, 3.0, m)))
+    x0 = torch.from_numpy(rng.poisson(100, n).astype(np.int32)).cuda()
+    out = {}
+
+    def run(lanes):
+        return lambda: api.simulate(net, x0, 1.0, n_traj, seed=7, max_events=500, lanes_per_traj=lanes, outputs=out)
+
+    assert ms(run(0)) <= 1.1 * ms(run(32))

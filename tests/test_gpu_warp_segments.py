@@ -66,3 +66,16 @@ def test_fewer_warps_per_block_and_no_moment_table(m, n, t_end):
     assert np.array_equal(a["grid_sum"].cpu().numpy(), np.where(known[..., None], grid, 0).sum(0))
     assert np.array_equal(a["grid_sumsq"].cpu().numpy(), np.where(known[..., None], grid * grid, 0).sum(0))
     assert np.array_equal(a["grid_count"].cpu().numpy(), known.sum(0))
+
+
+@pytest.mark.parametrize("m,n,n_traj", [(20, 5, 152 * 12), (20, 5, 152 * 12 + 1), (90, 20, 152 * 12 + 1),
+                                        (64, 2700, 1900), (64, 3300, 1900), (20, 12000, 1900), (100, 12000, 30)])
+def test_ramped_widths_by_trajectories_and_species(m, n, n_traj):
+    """Both sides of the lines between 32 lanes and the width by M: few trajectories, many species."""
+    net = W.random_mass_action(n, m, 7 + m, 0.5)
+    beta = np.where(np.arange(m) % 3 == 0, 0.0, 0.4)
+    x0 = np.random.default_rng(n).poisson(20, n).astype(np.int32)
+    kw = dict(seed=9, max_events=40)
+    g = api.simulate(api.Network(net).set_rate_slopes(beta), x0, 0.5, n_traj, grad=True, mapping=L.RT_MAP_WARP, **kw)
+    o = oracle.run(net, x0, 0.5, n_traj, beta=beta, want_grad=True, n_threads=8, **kw)
+    assert_same(g, o)
