@@ -354,7 +354,7 @@ static cudaError_t launch_rgc(const RunArgs &a, cudaStream_t s, int tend_finite)
   if (warp_state_off(a.net.M, nv, (int64_t)(mom / 8), TD, COPY) + per_warp > kWarpSmemMax) mom = 0;  // added in global memory
   const size_t off = warp_state_off(a.net.M, nv, (int64_t)(mom / 8), TD, COPY);
   int wpb = kWarpBlock / 32;  // fewer warps per block where many species or moments leave no room
-  while (wpb > 1 && off + wpb * per_warp > kWarpSmemMax) wpb /= 2;
+  while (wpb > 1 && off + wpb * per_warp > kWarpSmemMax) --wpb;
   const size_t smem = off + wpb * per_warp;
   const int64_t per_block = (int64_t)wpb * S;
   if ((a.n_traj + per_block - 1) / per_block > INT_MAX) return cudaErrorInvalidConfiguration;

@@ -79,3 +79,69 @@ def test_ramped_widths_by_trajectories_and_species(m, n, n_traj):
     g = api.simulate(api.Network(net).set_rate_slopes(beta), x0, 0.5, n_traj, grad=True, mapping=L.RT_MAP_WARP, **kw)
     o = oracle.run(net, x0, 0.5, n_traj, beta=beta, want_grad=True, n_threads=8, **kw)
     assert_same(g, o)
+
+
+def _warp_block_bytes(net, lanes, td, moments, warps):
+    """Shared memory of a block of `warps` warps, from the layout of the kernel: tables, moments, trajectories."""
+    m, n, nv = net.n_reactions, net.n_species, 0 if td else len(net.stoi_delta)
+    off = m * (24 if td else 16) + nv * 8 + moments + (0 if td else (m + 1) * 4)
+    off = (off + 127) // 128 * 128
+    pad = (m + lanes - 1) // lanes * lanes
+    seg = (pad * 36 + n * 4 + 63) // 128 * 128 + 64
+    return off + warps * (32 // lanes) * seg
+
+
+BLOCK_MAX = 226 * 1024
+
+
+@pytest.mark.parametrize("m,n,points,warps,table", [(64, 3050, 0, 3, False), (64, 3050, 1, 3, True), (60, 3060, 0, 3, False),
+                                                    (64, 2300, 1, 4, True), (128, 5600, 0, 4, False),
+                                                    (64, 3050, 2, 3, False)])
+def test_blocks_of_three_warps(m, n, points, warps, table):
+    """Blocks that four warps do not fit in, beside the largest that they do, with a moment table and without
+    (a table above 64 KB is left in global memory)."""
+    lanes = 8 if m <= 64 else 16
+    net = W.random_mass_action(n, m, 43 + m, 0.5)
+    tab = points * n * 16 + points * 8
+    tab = tab if tab <= 64 * 1024 else 0
+    assert (tab > 0) == table
+    assert _warp_block_bytes(net, lanes, False, tab, warps) <= BLOCK_MAX
+    assert warps == 4 or _warp_block_bytes(net, lanes, False, tab, warps + 1) > BLOCK_MAX
+    x0 = np.random.default_rng(n).poisson(15, n).astype(np.int32)
+    t_end = 0.5
+    kw = dict(seed=6, max_events=60, sample_dt=1.0 if points <= 1 else t_end / (points - 1))
+    g = api.simulate(api.Network(net), x0, t_end, 50, grad=True, grid="moments" if points else "none",
+                     mapping=L.RT_MAP_WARP, **kw)
+    o = oracle.run(net, x0, t_end, 50, want_grad=True, want_grid=points > 0, n_threads=8, **kw)
+    assert_same(g, o, ("x_final", "n_events", "status", "counts", "t_last", "t_internal", "loglik"))
+    if points:
+        grid = o["grid"].astype(np.int64)
+        known = (grid >= 0).all(axis=2)
+        assert grid.shape[1] == points
+        assert np.array_equal(g["grid_sum"].cpu().numpy(), np.where(known[..., None], grid, 0).sum(0))
+        assert np.array_equal(g["grid_sumsq"].cpu().numpy(), np.where(known[..., None], grid * grid, 0).sum(0))
+        assert np.array_equal(g["grid_count"].cpu().numpy(), known.sum(0))
+
+
+def test_moment_table_dropped_where_the_net_changes_fill_the_block():
+    """Reactions that change every species: with their net changes in shared memory a moment table that would
+    do by itself leaves no room for one warp, and the moments are added in global memory."""
+    m, n, points = 64, 320, 12
+    base = W.random_mass_action(n, m, 5, 0.5)
+    rng = np.random.default_rng(8)
+    net = W.Network(n, m, base.reac_rxn, base.reac_sp, base.reac_coef, np.repeat(np.arange(m), n),
+                    np.tile(np.arange(n), m), rng.choice([-1, 1], n * m), base.c)
+    tab = points * n * 16 + points * 8
+    assert tab <= 64 * 1024 and _warp_block_bytes(net, 8, False, tab, 1) > BLOCK_MAX
+    assert _warp_block_bytes(net, 8, False, 0, 4) <= BLOCK_MAX
+    x0 = np.full(n, 200, np.int32)
+    kw = dict(seed=6, max_events=60, sample_dt=1e-6)
+    g = api.simulate(api.Network(net), x0, 1.1e-5, 70, grad=True, grid="moments", mapping=L.RT_MAP_WARP, **kw)
+    o = oracle.run(net, x0, 1.1e-5, 70, want_grad=True, want_grid=True, n_threads=8, **kw)
+    assert o["n_events"].max() > 5 and o["grid"].shape[1] == points
+    assert_same(g, o, ("x_final", "n_events", "status", "counts", "t_last", "t_internal", "loglik"))
+    grid = o["grid"].astype(np.int64)
+    known = (grid >= 0).all(axis=2)
+    assert np.array_equal(g["grid_sum"].cpu().numpy(), np.where(known[..., None], grid, 0).sum(0))
+    assert np.array_equal(g["grid_sumsq"].cpu().numpy(), np.where(known[..., None], grid * grid, 0).sum(0))
+    assert np.array_equal(g["grid_count"].cpu().numpy(), known.sum(0))
