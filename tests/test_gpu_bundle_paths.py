@@ -69,3 +69,18 @@ def test_every_lane_reads_the_partials_of_its_event(ctas):
     of an earlier event would leave the oracle's path."""
     net = W.random_mass_action(600, 152 * 32, 77, 1.0)
     check(net, W.poisson_x0(600, 40, 5), n_traj=1 if ctas > 76 else 2, max_events=2000, ctas_per_traj=ctas)
+
+
+def test_every_trajectory_stops_at_the_range_check():
+    """One channel fires up to the last count that fits and is not fired past it, in every trajectory."""
+    m = 300
+    base = W.random_mass_action(40, m, 12, 0.5)
+    c = np.full(m, 1e-12)
+    k = int(base.stoi_rxn[base.stoi_delta > 0][0])
+    s = int(base.stoi_sp[base.stoi_delta > 0][0])
+    c[k] = 1.0
+    x0 = np.full(40, 1000, np.int32)
+    x0[s] = 2**31 - 5
+    o = check(base.with_rates(c), x0, max_events=50, ctas_per_traj=2)
+    assert (o["status"] == oracle.ST_OVERFLOW).all()
+    assert (o["n_events"] > 0).all() and (o["n_events"] < 50).all()

@@ -65,3 +65,31 @@ def test_one_channel_again_and_again():
     c[137] = 5.0
     check(net.with_rates(c), np.full(20, 500, np.int32), max_events=400)
     check(W.pure_birth(3.0), np.zeros(1, np.int32), max_events=300)
+
+
+def _list_bytes(net, ctas):
+    """Shared memory of a slice with the event's list of touched channels once per channel and once per reader
+    list, from the sizes the kernel's plan is made of (16 bytes a group, 40 an entry, X)."""
+    readers = np.bincount([s for _, s in set(zip(net.reac_rxn.tolist(), net.reac_sp.tolist()))],
+                          minlength=net.n_species)
+    change = {}
+    for r, s, d in zip(net.stoi_rxn.tolist(), net.stoi_sp.tolist(), net.stoi_delta.tolist()):
+        change[r, s] = change.get((r, s), 0) + d
+    dep = np.zeros(net.n_reactions, np.int64)
+    for (r, s), d in change.items():
+        if d:
+            dep[r] += readers[s]
+    chunk = (-(-net.n_reactions // ctas) + 31) // 32 * 32
+    most = int(dep.max())
+    assert api.Network(net).info()["max_dependents"] == most
+    return [chunk // 32 * 16 + cap * 40 + net.n_species * 4 for cap in (min(chunk, most + 1), min(2 * chunk, most) + 1)]
+
+
+@pytest.mark.parametrize("m,n,ctas", [(4400, 2, 1), (4900, 3, 1), (9000, 2, 2)])
+def test_list_that_fits_once_per_channel_only(m, n, ctas):
+    """Networks so dense that an event's list has no room for a channel found in two reader lists: each channel is
+    updated where it is found and takes its entry there."""
+    net = W.random_mass_action(n, m, 6, 0.5)
+    once, twice = _list_bytes(net, ctas)
+    assert once <= 200 * 1024 < twice
+    check(net, W.poisson_x0(n, 40, 3), n_traj=2, max_events=80, ctas_per_traj=ctas, grad=ctas == 1)
