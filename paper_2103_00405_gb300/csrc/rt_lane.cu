@@ -241,9 +241,12 @@ constexpr int64_t kLaneFp64Traj = 152 * 8;
 // ensemble sizes at which one thread per trajectory overtakes it.  Measured, lane / thread: Lotka-Volterra
 // 64 trajectories 5.1 / 17.0 ms, 3000 9.8 / 17.9 ms, 8000 25.8 / 18.3 ms; birth-death 64 0.62 / 1.53 ms,
 // 3000 1.18 / 1.60 ms, 4000 1.65 / 1.64 ms; 12 reactions 64 1.0 / 8.0 ms, 8000 4.7 / 8.1 ms,
-// 16000 8.6 / 8.6 ms; 16 reactions 8000 16.7 / 27 ms, 16000 30 / 28 ms.
+// 16000 8.6 / 8.6 ms; 16 reactions 8000 16.7 / 27 ms, 16000 30 / 28 ms.  A thread's event takes longer with M, a
+// warp's does not.  Time of the thread kernel over the lane kernel's, three networks each, at 152 x 64 / 152 x 72
+// trajectories: 5 reactions 0.90, 1.10, 1.07 / 0.80, 0.98, 0.91; 6 reactions 1.15, 1.27, 1.06 / 1.02, 1.11, 0.92;
+// 7 reactions 1.08, 1.19, 1.17 / 0.95, 1.06, 1.03; 8 and 9 at least 1.21 / 1.08.
 bool lane_mapping_fits(const DevNet &net, int64_t n_traj) {
-  return net.M <= kLaneMaxM && net.N <= kLaneMaxN && n_traj <= (net.M <= 4 ? 152 * 24 : 152 * 72);
+  return net.M <= kLaneMaxM && net.N <= kLaneMaxN && n_traj <= 152 * (net.M <= 4 ? 24 : net.M == 5 ? 64 : 72);
 }
 
 template <int MP>

@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():  # pragma: no cover - CPU-only hosts skip the GPU suite
     pytest.skip("CUDA not available", allow_module_level=True)
 
+from paper_2103_00405_gb300 import _lib as L  # noqa: E402
 from paper_2103_00405_gb300 import api  # noqa: E402
 
 
@@ -42,3 +43,16 @@ def test_ramped_segment_width_by_trajectories(m, n_traj):
         return lambda: api.simulate(net, x0, 1.0, n_traj, seed=7, max_events=500, lanes_per_traj=lanes, outputs=out)
 
     assert ms(run(0)) <= 1.1 * ms(run(32))
+
+
+@pytest.mark.parametrize("m,n_traj", [(3, 152 * 23), (5, 152 * 40), (5, 152 * 70), (8, 152 * 71), (12, 152 * 71)])
+def test_few_trajectories_of_a_small_network(m, n_traj):
+    n = 6
+    net = api.Network(W.random_mass_action(n, m, W.GEN_SEED_BASE + m, 0.5))
+    x0 = torch.from_numpy(np.random.default_rng(m).poisson(200, n).astype(np.int32)).cuda()
+    out = {}
+
+    def run(mapping):
+        return lambda: api.simulate(net, x0, 2.0, n_traj, seed=7, max_events=600, mapping=mapping, outputs=out)
+
+    assert ms(run(None)) <= 1.1 * ms(run(L.RT_MAP_THREAD))

@@ -63,6 +63,15 @@ def test_choice_does_not_change_results(m, n, n_traj):
     same(a, b, KEYS + ("grid_sum", "grid_sumsq", "grid_count"))
 
 
+@pytest.mark.parametrize("n_traj", [9728, 9729])
+def test_choice_at_five_reactions(n_traj):
+    net = net_of(5, 4)
+    x0 = np.random.default_rng(3).integers(0, 90, (n_traj, 4)).astype(np.int32)
+    kw = dict(seed=4, max_events=60, grad=True)
+    same(api.simulate(api.Network(net), x0, 0.5, n_traj, **kw),
+         api.simulate(api.Network(net), x0, 0.5, n_traj, mapping=L.RT_MAP_THREAD, **kw), KEYS)
+
+
 @pytest.mark.parametrize("n_traj", [3, 20000])
 def test_forbidden_channels_overflow_and_absorption(n_traj):
     spec = W.Network(3, 6, [1, 2, 3, 4, 5], [0, 1, 0, 2, 2], [1, 1, 2, 1, 1], [0, 1, 1, 3, 5], [0, 0, 1, 2, 2],
