@@ -2,8 +2,9 @@
 
 Batched mode: the class thresholds (thread / warp / block per trajectory) and the
 block size of the persistent kernel decide how thousands of uneven networks share
-the GPU.  Single networks: the mapping (thread, warp, block, bundle) and its block
-size.  Each candidate runs a short probe (a capped number of events per
+the GPU.  Single networks: what the library chooses by itself (from the network's size
+and the number of trajectories; some kernels and block sizes run only so) and each
+mapping (thread, warp, block, bundle) with its block sizes.  Each candidate runs a short probe (a capped number of events per
 trajectory, same networks and seeds) timed with CUDA events; the fastest in
 events per second wins.  Choices are cached in a JSON file keyed by GPU name and
 problem shape (``RANDTIME_AUTOTUNE_CACHE`` overrides the path).
@@ -110,6 +111,10 @@ def tune_batch(specs, x0: torch.Tensor, t_end: torch.Tensor, n_traj: int = 1, pr
     return best
 
 
+# the library's own choice of mapping and block size, which no named mapping stands for
+LIBRARY_CHOICE = dict(mapping=L.RT_MAP_AUTO, block_threads=0)
+
+
 def single_key(spec, n_traj: int) -> str:
     return "single|%s|M=%d|N=%d|traj=%d" % (_gpu(), spec.n_reactions, spec.n_species, n_traj)
 
@@ -120,10 +125,11 @@ def tune_single(spec, x0, t_end: float, n_traj: int, probe_events: int = 2000, u
     key = single_key(spec, n_traj)
     if use_cache:
         hit = _load_cache().get(key)
-        if hit:
+        # an entry that lists what it tried without the library's own choice is timed again
+        if hit and ("tried" not in hit or any(c == LIBRARY_CHOICE for c, _ in hit["tried"])):
             return hit["launch"]
     M = spec.n_reactions
-    cands = []
+    cands = [dict(LIBRARY_CHOICE)]
     if M <= 16:
         cands += [dict(mapping=L.RT_MAP_THREAD, block_threads=b) for b in (64, 128)]
     if M <= 256:
