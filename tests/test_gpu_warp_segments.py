@@ -124,13 +124,13 @@ def test_blocks_of_three_warps(m, n, points, warps, table):
 
 
 def test_moment_table_dropped_where_the_net_changes_fill_the_block():
-    """Reactions that change every species: with their net changes in shared memory a moment table that would
+    """Reactions that make some of every species: with their net changes in shared memory a moment table that would
     do by itself leaves no room for one warp, and the moments are added in global memory."""
     m, n, points = 64, 320, 12
     base = W.random_mass_action(n, m, 5, 0.5)
     rng = np.random.default_rng(8)
     net = W.Network(n, m, base.reac_rxn, base.reac_sp, base.reac_coef, np.repeat(np.arange(m), n),
-                    np.tile(np.arange(n), m), rng.choice([-1, 1], n * m), base.c)
+                    np.tile(np.arange(n), m), rng.integers(1, 3, n * m), base.c)
     tab = points * n * 16 + points * 8
     assert tab <= 64 * 1024 and _warp_block_bytes(net, 8, False, tab, 1) > BLOCK_MAX
     assert _warp_block_bytes(net, 8, False, 0, 4) <= BLOCK_MAX
