@@ -800,7 +800,8 @@ static LazyPlan plan_lazy(const DevNet &net, int max_dependents, int64_t n_traj,
   p.compact = size(twice) <= smem_budget ? 1 : 0;
   p.cap = (int)(p.compact ? twice : once);
   const size_t base = size(p.cap);
-  p.sptr_smem = base + (size_t)(net.N + 1) * 4 <= smem_budget ? 1 : 0;
+  // the species offsets are read only where reactions have no dependency records
+  p.sptr_smem = !net.vdep && base + (size_t)(net.N + 1) * 4 <= smem_budget ? 1 : 0;
   p.smem = base + (p.sptr_smem ? (size_t)(net.N + 1) * 4 : 0);
   return p;
 }
