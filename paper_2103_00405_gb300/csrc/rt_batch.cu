@@ -5,8 +5,9 @@
 // class by size (thread, warp or block per trajectory).  The flattened work list
 // is (network rank in its class, trajectory), networks sorted by decreasing size
 // so the longest items start first; it is cut into block-sized tasks: one
-// block-class trajectory, block_threads/32 warp-class trajectories or
-// block_threads thread-class trajectories.  Persistent blocks take tasks from an
+// block-class trajectory, one warp-class trajectory per warp (fewer where the
+// largest one's state would keep a second block off the SM) or block_threads
+// thread-class trajectories.  Persistent blocks take tasks from an
 // atomic counter and run the same per-trajectory routines as the single-network
 // kernels (rt_traj_*.cuh), reading the network tables through generic pointers
 // into the arena.  Network i uses its own Philox stream (the fourth counter word;
@@ -88,11 +89,11 @@ __device__ __forceinline__ RunArgs item_args(const BatchArgs &B, int net_index, 
   return A;
 }
 
-// Two resident blocks per SM (64 registers; the block routine's channel state partly
-// spills to L1-backed local memory): a block-class trajectory is latency-bound (barriers,
-// dependent loads, one thread's Exp(1) draw per event), and a second block on the SM
-// runs while the first waits -- measured 1.28x the single-block kernel on the 4096-network
-// batch.
+// Two resident blocks per SM (64 registers; the block routine keeps T in them, propensities
+// and float bounds in shared memory): a block-class trajectory is latency-bound (three
+// barriers per event, a short chain behind each), and a second block on the SM runs while
+// the first waits -- measured 1.28x the single-block kernel on the 4096-network batch, with
+// the routine as it was when its state was in registers.
 template <bool LL>
 __global__ void __launch_bounds__(512, 2) k_batch(const BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem[];

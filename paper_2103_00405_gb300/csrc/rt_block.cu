@@ -1,6 +1,8 @@
 // rt_block.cu -- one thread block per trajectory (RT_MAP_BLOCK): the single-network
 // kernel around block_trajectory (rt_traj_block.cuh), for networks of up to
-// 8 * block_threads reactions with all per-channel state in registers.
+// 8 * block_threads reactions: T in registers, propensities and float bounds in shared
+// memory (in local memory where many species leave no room), P and the next increments in
+// local memory.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -664,7 +664,7 @@ int launch_bundle_mapping(const RunArgs &a, int ctas_per_traj, void *ws, size_t 
   B.tend_finite = std::isfinite(a.t_end) ? 1 : 0;
   B.want_T = (a.out.t_internal_dev || a.out.loglik_dev) ? 1 : 0;
   B.depth = p.depth;
-  long long spin = 20000000;  // ~2 s of 100 ns polls
+  long long spin = 20000000;  // polls, with a sleep of about a microsecond each after the first 256: 20 to 30 s
   if (const char *env = getenv("RT_DEBUG_SPIN_LIMIT")) spin = atoll(env);
   B.spin_limit = spin;
   B.traj0 = 0;

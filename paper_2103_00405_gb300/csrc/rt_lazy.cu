@@ -27,8 +27,9 @@
 //   4. updates the minima of the 32-channel groups that hold a touched channel (one thread per
 //      group; a group whose minimum was touched re-reads its untouched channels, one warp each).
 // What bounds it is latency: an event is a chain of memory (1500 cycles a miss; the records of 16
-// trajectories of 10^6 channels are 512 MB), barriers and 64-cycle FP64 operations, under 1 % of the
-// memory's rate.  Per event at that size 7.9 us when one thread polled, decided and wrote the decision
+// trajectories of 10^6 channels are 512 MB), barriers and 64-cycle FP64 operations.  It moves 153 KB per
+// event (104 KB before the prefetch for the second candidate; 42 KB by count), 6.6 % of the memory's rate.
+// Per event at that size 7.9 us when one thread polled, decided and wrote the decision
 // for the others and every touched channel was loaded in three dependent steps and divided on the
 // FP64 pipe; 6.8 us without those, 6.4 us with packed lists, 5.5 us with the prefetch.
 // Ties go to the smallest index at every level, so the minimum is the exact one.
@@ -908,7 +909,8 @@ int launch_lazy_mapping(const RunArgs &a, int max_dependents, int ctas_per_traj,
   L.sptr_smem = p.sptr_smem;
   L.tend_finite = std::isfinite(a.t_end) ? 1 : 0;
   L.want_T = (a.out.t_internal_dev || a.out.loglik_dev) ? 1 : 0;
-  long long spin = 20000000;  // polls before a trajectory gives up (each a few tens of ns)
+  // polls before a trajectory gives up, with a sleep of about a microsecond each after the first 4096: some 20 s
+  long long spin = 20000000;
   if (const char *env = getenv("RT_DEBUG_SPIN_LIMIT")) spin = atoll(env);
   L.spin_limit = spin;
   k_lazy_init<<<152 * 8, 256, 0, s>>>(L);

@@ -5,7 +5,7 @@
 // spread over the G lanes of its segment (Eq. 17-27).  Only the internal times T_k live in
 // registers; P_k, a_k, the increment drawn ahead for the channel's next firing, its firing
 // count and two floats (an upper bound of P_k, and of 1 / a_k) are in shared memory, so that
-// the state of eight channels per lane leaves room for six blocks of four warps per SM, and so
+// with eight channels per lane five or six blocks of four warps fit on an SM, and so
 // that the propensities an event changed can be recomputed by any lane of the segment: its
 // list of dependent channels is dealt out to the lanes one each.
 //

@@ -28,13 +28,15 @@ __host__ __device__ inline size_t warp_state_off(int M, int nv, int64_t nmom, bo
   return (b + 127) / 128 * 128;
 }
 
-// Registers bounded (80) for six blocks, 24 warps, per SM.  Against the state in registers (128, 16 warps):
-// 65536 trajectories of 64 reactions with likelihood and gradient 350 -> 186 ms, 10000 trajectories of 200
-// reactions with moments 74.8 -> 51.8 ms; time-dependent rates against every root exactly with one
-// trajectory per warp: 10000 trajectories of 48 reactions 83 -> 26 ms.
+// Registers bounded (80) for six blocks, 24 warps, per SM; shared memory (one KB of a block is the system's)
+// may hold fewer: 64 reactions with 16 species 40.3 KB a block, 5 blocks; 200 reactions with 50 species 6, with
+// the moments of 21 grid points (53.8 KB) 4.  Against the state in registers (128, 16 warps): 65536 trajectories
+// of 64 reactions with likelihood and gradient 350 -> 181 ms, 10000 trajectories of 200 reactions with moments
+// 74.8 -> 47.6 ms; time-dependent rates against every root exactly with one trajectory per warp: 10000
+// trajectories of 48 reactions 83 -> 25 ms.
 // COPY: the net changes in shared memory too (else, read once per event, in global memory: where their
-// copies would keep a block off the SM -- 200 reactions, 5 instead of 6 blocks, 47.6 -> 45.5 ms; with
-// the blocks that fit unchanged the copies are the better place, 64 reactions 180 against 207 ms).
+// copies would keep a block off the SM -- those 200 reactions with moments, 3 instead of 4 blocks, 47.6 ->
+// 45.4 ms; with the blocks that fit unchanged the copies are the better place, 64 reactions 180 against 207 ms).
 template <int R, int G, bool LL, bool TD, bool COPY>
 __global__ void __launch_bounds__(kWarpBlock, 6)
     k_ens_warp(const RunArgs A, const int tend_finite, const int use_mom) {
@@ -377,7 +379,10 @@ static int blocks_that_fit(const RunArgs &a, bool copy) {
 
 template <int R, int G, bool TD>
 static cudaError_t launch_rg(const RunArgs &a, cudaStream_t s, int tf) {
-  // only the widest networks' copies can cost a block; TD's net changes may not fit at all
+  // The rule is kept to the widest networks.  Moments' tables can make the copies cost a block below them too, and
+  // there it goes both ways (21 grid points, 10000 / 30000 trajectories, copies against none): 64 reactions 2.85 /
+  // 6.08 against 2.00 / 5.54 ms, 104 reactions 3.75 / 9.06 against 3.18 / 8.57, but 84 reactions 2.88 / 7.68 against
+  // 3.11 / 8.24.  TD's net changes may not fit at all.
   if constexpr (TD || (R == 8 && G == 32)) {
     if (TD || blocks_that_fit<G, TD>(a, true) < blocks_that_fit<G, TD>(a, false))
       return launch_rgc<R, G, TD, false>(a, s, tf);
@@ -413,7 +418,9 @@ static int choose_lanes(int M, int requested) {
   return M <= 64 ? 8 : M <= 128 ? 16 : 32;
 }
 
-// Shared memory one warp of a block needs, its block's tables included: what a network must fit in.
+// What decides whether a network is refused: its tables, a byte per channel and lane, and four warps' X within
+// 200 KB.  Above that limit stands what a block really holds (warp_state_off, warp_seg_bytes): one warp of every
+// network within it fits (at most 10 KB more), and launch_rgc takes as many as do.
 static size_t warp_fit_bytes(const DevNet &d, int G) {
   return (size_t)d.M * (8 + 8) + (size_t)d.n_vnz * 8 + (size_t)(d.M + 1) * 4 + (((size_t)d.M * G + 15) & ~(size_t)15) +
          (size_t)d.N * 4 * (kWarpBlock / 32) * (32 / G);
