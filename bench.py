@@ -63,8 +63,9 @@ FP64_OP_NOMINAL = 0.625e12
 NCU_TRAFFIC = {
     "k_bundle": dict(bytes_per_unit=(19653502208 + 7660353792) / (60 * 16 * 1e6), unit="channel-event",
                      source="ncu capture of k_bundle<false>, N=1e4, M=1e6, 16 trajectories x 60 events"),
-    "k_ens_small": dict(bytes_per_unit=(818944 + 0) / 16384, unit="trajectory",
-                        source="ncu capture of k_ens_small<3,2,false>, 16384 Lotka-Volterra trajectories to t=10"),
+    "k_ens_small": dict(bytes_per_unit=(196864 + 44288) / 1048576, unit="trajectory",
+                        source="ncu capture of k_ens_small<3,2,false>, 2^20 Lotka-Volterra trajectories to t=0.1 "
+                               "(outputs stay in L2)"),
     "k_lazy": dict(bytes_per_unit=(3024477696 + 649416448) / (16 * 1500), unit="event",
                    source="ncu capture of k_lazy<false, true>, N=1e4, M=1e6, 16 trajectories x 1500 events"),
 }
@@ -638,12 +639,12 @@ def run_large_tree(args, ctx, steps, warmup):
                          "traffic": (NCU_TRAFFIC["k_lazy"]["bytes_per_unit"] * events / steps
                                      if NCU_TRAFFIC["k_lazy"]["bytes_per_unit"] else None),
                          "traffic_note": NCU_TRAFFIC["k_lazy"]["source"] + ", scaled to this launch's events (random "
-                                         "32-byte sectors: ~2.5x the algorithmic bytes)",
-                         "kernel": "k_lazy<false>", "bytes_per_event": bytes_per_event,
+                                         "32-byte sectors and prefetches: ~3.7x the algorithmic bytes)",
+                         "kernel": "k_lazy<false, true>", "bytes_per_event": bytes_per_event,
                          "touched_channels_per_event": touched, "peak_source": how,
                          "note": "latency-bound: each event is a chain of dependent steps (slice minima, mailbox "
                                  "exchange, fire, touched channels, group minima); the bytes moved per event are "
-                                 "under 1/700 of the internal-time scan's 32 MB, so the HBM fraction is small by "
+                                 "under 1/600 of the internal-time scan's 28 MB, so the HBM fraction is small by "
                                  "construction; the event rate is the figure of merit"}}
 
 
@@ -701,7 +702,7 @@ def run_table3(args, ctx, steps, warmup):
         dev_ms, events_all = combine_over_ranks(sum(ms), sum(step_events), ctx.world, ctx.dev)
         mid[name] = {"value": events_all / (dev_ms / 1e3), "unit": UNIT, "ms_per_step": dev_ms / steps,
                      "kernel": "k_ens_rescaled_warp<2,false>" if form == L.RT_FORM_RESCALED
-                     else "k_ens_warp<8,8,false>"}
+                     else "k_ens_warp<8,8,false,false,true>"}
     line = {"value": res["table3_rescaled"]["value"], "unit": UNIT, "steps": steps, "warmup": warmup,
             "ms_per_step": res["table3_rescaled"]["ms_per_step"],
             "config": {"workload": "Table 3's form vs Table 2's internal-time form: Lotka-Volterra (Fig. 1 model, "
@@ -852,7 +853,8 @@ def run_grad(args, ctx, steps, warmup):
     counts = out_grad["counts"].sum(0, dtype=torch.int64).cpu().numpy()
     ops, ev = fp64_ops_per_event(net, counts, 2)
     fwd_ms = statistics.mean(m["forward"] for m in marks)
-    roof = alu_roofline(ops, fwd_ms, ctx.fp64_peak, "k_ens_warp<8,8,true> (8 lanes per trajectory, forward with the log-likelihood)",
+    roof = alu_roofline(ops, fwd_ms, ctx.fp64_peak,
+                        "k_ens_warp<8,8,true,false,true> (8 lanes per trajectory, forward with the log-likelihood)",
                         "%.1f FP64 ops per event (2M+2; quotients, propensities and logarithms are integer "
                         "work)" % (ops / ev))
     return {"value": events_all / (dev_ms / 1e3), "unit": UNIT, "steps": steps, "warmup": warmup,
@@ -862,7 +864,7 @@ def run_grad(args, ctx, steps, warmup):
                                    % cfg["n_traj"],
                        "parallelism": ("trajectories sharded over %d ranks, grad_c summed in rank order"
                                        % ctx.world) if ctx.world > 1 else "1 GPU",
-                       "l2": "state in registers; outputs 64 MB written per step"},
+                       "l2": "state on chip; outputs 64 MB written per step"},
             "events_per_step": events_all / steps, "clocks": clocks, "gpu_launches": 2 * steps,
             "backward_ms": statistics.mean(m_ - m["forward"] for m_, m in zip(ms, marks)),
             "roofline": roof,
