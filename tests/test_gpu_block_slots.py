@@ -78,3 +78,24 @@ def test_species_limit_does_not_depend_on_the_trajectories(n_traj):
     wide = W.random_mass_action(n + 1, m, 71, 0.7)
     with pytest.raises(L.RandtimeError):
         api.simulate(api.Network(wide), np.zeros(n + 1, np.int32), 1.0, n_traj, **kw)
+
+
+@pytest.mark.parametrize("m,tiny", [(600, 6), (600, 7), (600, 8), (600, 9), (600, 31), (600, 33), (600, 599), (2000, 1500),
+                                    (300, 40)])
+@pytest.mark.parametrize("rate", [1e-45, 1e-320, 1e40])
+def test_many_candidates(m, tiny, rate):
+    """Channels whose rates no float bound covers are candidates of every event: lists of a few, of more than a
+    warp, and of every channel."""
+    n = m // 4
+    net = W.random_mass_action(n, m, 81, 0.7)
+    c = net.c.copy()
+    if rate > 1:
+        c *= rate
+    c[np.random.default_rng(m + tiny).permutation(m)[:tiny]] = rate
+    x0 = np.random.default_rng(m).poisson(60, n).astype(np.int32)
+    t_end = 1e-30 if rate > 1 else 1e6
+    kw = dict(seed=11, max_events=120)
+    for n_traj in (2, 700 if m == 300 else 3):  # a block of one slot per thread, and of several
+        g = api.simulate(api.Network(net.with_rates(c)), x0, t_end, n_traj, grad=True, mapping=L.RT_MAP_BLOCK, **kw)
+        o = oracle.run(net.with_rates(c), x0, t_end, n_traj, want_grad=True, n_threads=8, **kw)
+        assert_same(g, o)

@@ -56,3 +56,20 @@ def test_few_trajectories_of_a_small_network(m, n_traj):
         return lambda: api.simulate(net, x0, 2.0, n_traj, seed=7, max_events=600, mapping=mapping, outputs=out)
 
     assert ms(run(None)) <= 1.1 * ms(run(L.RT_MAP_THREAD))
+
+
+def test_rates_that_no_float_bound_covers():
+    """A third of the channels with rates of 1e-45: every one is computed exactly at every event, which may cost
+    as much again as the event and half as much more, not several times it."""
+    m, n = 3000, 750
+    spec = W.random_mass_action(n, m, W.GEN_SEED_BASE + m, 0.5)
+    x0 = torch.from_numpy(np.random.default_rng(m).poisson(100, n).astype(np.int32)).cuda()
+    out = {}
+
+    def run(rate):
+        c = spec.c.copy()
+        c[-m // 3:] = rate
+        net = api.Network(spec.with_rates(c))
+        return lambda: api.simulate(net, x0, 1e6, 64, seed=7, max_events=500, outputs=out)
+
+    assert ms(run(1e-45)) <= 2.5 * ms(run(1e-12))
