@@ -31,7 +31,7 @@ __host__ __device__ inline size_t warp_state_off(int M, int nv, int64_t nmom, bo
 // Registers bounded (80) for six blocks, 24 warps, per SM; shared memory (one KB of a block is the system's)
 // may hold fewer: 64 reactions with 16 species 40.3 KB a block, 5 blocks; 200 reactions with 50 species 6, with
 // the moments of 21 grid points (53.8 KB) 4.  Against the state in registers (128, 16 warps): 65536 trajectories
-// of 64 reactions with likelihood and gradient 350 -> 181 ms, 10000 trajectories of 200 reactions with moments
+// of 64 reactions with likelihood and gradient 350 -> 169 ms, 10000 trajectories of 200 reactions with moments
 // 74.8 -> 47.6 ms; time-dependent rates against every root exactly with one trajectory per warp: 10000
 // trajectories of 48 reactions 83 -> 25 ms.
 // COPY: the net changes in shared memory too (else, read once per event, in global memory: where their

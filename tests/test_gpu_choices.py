@@ -73,3 +73,17 @@ def test_rates_that_no_float_bound_covers():
         return lambda: api.simulate(net, x0, 1e6, 64, seed=7, max_events=500, outputs=out)
 
     assert ms(run(1e-45)) <= 2.5 * ms(run(1e-12))
+
+
+@pytest.mark.parametrize("m", [64, 128, 200, 256])
+def test_runs_that_fire_no_event(m):
+    """The increments of the next firings are not drawn before one is needed: a run that stops before its first
+    event takes at most six tenths of one with ten events."""
+    net = api.Network(W.random_mass_action(m // 4, m, W.GEN_SEED_BASE + m, 0.5))
+    x0 = torch.from_numpy(np.random.default_rng(m).poisson(100, m // 4).astype(np.int32)).cuda()
+    out = {}
+
+    def run(events):
+        return lambda: api.simulate(net, x0, 5.0, 100000, seed=7, max_events=events, outputs=out)
+
+    assert ms(run(0)) <= 0.6 * ms(run(10))
